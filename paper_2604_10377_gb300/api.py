@@ -462,13 +462,16 @@ def overlap_metrics(scores: torch.Tensor, labels: torch.Tensor, seg_offsets, thr
         raise ValueError("scores and labels must be contiguous and of equal length")
     off = np.asarray(seg_offsets, dtype=np.int64)
     n_seg = len(off) - 1
-    if n_seg < 0 or (n_seg > 0 and (off[0] < 0 or np.any(np.diff(off) < 0) or off[-1] > scores.numel())):
+    lengths = np.diff(off)
+    if n_seg < 0 or (n_seg > 0 and (off[0] < 0 or lengths.min() < 0 or off[-1] > scores.numel())):
         raise ValueError("seg_offsets must be non-decreasing offsets within the arrays")
     dev = scores.device
     counts = torch.empty((max(n_seg, 1), 4), dtype=torch.int64, device=dev)
     metrics = torch.empty((max(n_seg, 1), 7), dtype=torch.float64, device=dev) if with_metrics else None
+    max_len = int(lengths.max()) if n_seg > 0 else 0
+    # the copy of the offsets waits for the stream's earlier work: everything else comes before it,
+    # so that the GPU idles only for the copy and the launches
     off_dev = torch.from_numpy(off).to(dev)
-    max_len = int(np.max(np.diff(off))) if n_seg > 0 else 0
     check(_lib.lib().fmap_overlap_metrics(_ptr(scores), _ptr(labels), _ptr(off_dev), n_seg, max_len,
                                           float(threshold), _ptr(counts), _ptr(metrics), _stream(dev)),
           "fmap_overlap_metrics")
