@@ -82,13 +82,13 @@ typedef struct fmap_options {
     int32_t bwd_chunk_v;        /* tensor-core backward projection: largest vertex chunk of a work
                                    item, multiple of 128 in 1024..65536 (default 8192) */
     int32_t solve_threads_k64;  /* row-solve block for k <= 64: 64 or 128 threads (default 64) */
-    int32_t solve_threads_k128; /* row-solve block for 64 < k <= 128: 128 or 256 (default 128) */
+    int32_t solve_threads_k128; /* row-solve block for 64 < k <= 100: 128 or 256 (default 128) */
     /* Persistent CTAs of the tensor-core projections, 1..152 (0 = one per SM, 152). A batch
      * whose projection runs beside another batch's row solves (two streams) can keep it on
      * part of the SMs, so that the solves' blocks hold the rest. */
     int32_t proj_ctas;          /* forward projection */
     int32_t bwd_ctas;           /* backward projection, even (two CTAs share each vertex tile) */
-    int32_t solve_no_g_copy;    /* row solves of k <= 128: 0 keeps a copy of G in shared memory for the
+    int32_t solve_no_g_copy;    /* row solves of k <= 100: 0 keeps a copy of G in shared memory for the
                                    refinement residual (default), 1 reads G from L2 instead (less shared
                                    memory per block, more blocks per SM) */
     int32_t adjoint_kernel;     /* W = Gamma^T C + C^T Gamma, dA_x = Gamma^T A_y - W A_x, dA_y = Gamma A_x,

@@ -508,22 +508,19 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
     P.shapes[s].slot_end = (int32_t)P.slot_list.size();
   }
 
-  // ---- row systems, grouped by block size, largest k first
-  // (k <= 64: 64 threads, <= 128: 128, <= 256: 256, <= kMaxK: 320 -- every block has at
-  // least one thread per padded row)
-  const int bounds[4] = {64, 128, 256, kMaxK};
-  const int threads[4] = {opt.solve_threads_k64 ? opt.solve_threads_k64 : 64,
-                          opt.solve_threads_k128 ? opt.solve_threads_k128 : 128, 256, 320};
-  for (int gi = 0; gi < 4; ++gi) {
+  // ---- row systems, grouped by class (kSolveBounds), largest k first
+  for (int gi = 0; gi < kSolveClasses; ++gi) {
     SolveGroup g{};
     g.first = (int32_t)P.systems.size();
-    g.threads = threads[gi];
+    // the knobs' block sizes of the first two classes (every block has a thread per padded row)
+    g.threads = gi == 0 ? (opt.solve_threads_k64 ? opt.solve_threads_k64 : 64)
+                        : (opt.solve_threads_k128 ? opt.solve_threads_k128 : 128);
     g.no_g_copy = opt.solve_no_g_copy;
     std::vector<int> members;
     for (int p = 0; p < n_pairs; ++p) {
       const int k = P.pairs[p].k;
-      const int lo = gi == 0 ? 0 : bounds[gi - 1];
-      if (k > lo && k <= bounds[gi]) members.push_back(p);
+      const int lo = gi == 0 ? 0 : kSolveBounds[gi - 1];
+      if (k > lo && k <= kSolveBounds[gi]) members.push_back(p);
     }
     std::stable_sort(members.begin(), members.end(), [&](int a, int b) { return P.pairs[a].k > P.pairs[b].k; });
     for (int p : members) {

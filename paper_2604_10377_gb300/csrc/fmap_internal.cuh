@@ -17,6 +17,9 @@ constexpr int kMaxK = 304;
 // per-pair partial sums of the training loss: one per 64 x 64 tile of C
 constexpr int kMaxLossTiles = ((kMaxK + 63) / 64) * ((kMaxK + 63) / 64);
 constexpr int kMaxD = 4096;
+// classes of the row solves by k_X (upper bounds): a launch each
+constexpr int kSolveClasses = 6;
+constexpr int kSolveBounds[kSolveClasses] = {64, 100, 128, 200, 208, kMaxK};
 
 // Device copy of a shape descriptor plus the offsets the library assigns to it.
 struct ShapeDev {
