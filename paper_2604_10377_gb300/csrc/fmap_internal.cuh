@@ -180,6 +180,7 @@ cudaError_t launch_project_tc_reduce(const ShapeDev* shapes, const TcItem* items
 
 // ---- launchers (each enqueues on `st`; return cudaError_t of the launch) ----
 // with_r = false computes G only (the adjoint solves never read R)
+cudaError_t gram_set_smem();
 cudaError_t launch_gram(const BatchDev& b, int max_k, const float* a, float* ws, cudaStream_t st,
                         bool with_r = true);
 

@@ -1255,6 +1255,7 @@ cudaError_t solve_set_smem_limits() {
   if ((e = set_limit(chol_reg_kernel<2, 2, 3, 4>, chol_reg_smem_bytes(kSolveBounds[2]))) != cudaSuccess) return e;
   if ((e = set_limit(chol_reg_kernel<5, 4, 2, 2>, chol_reg_smem_bytes(kSolveBounds[3]))) != cudaSuccess) return e;
   if ((e = set_limit(chol_reg_kernel<14, 5, 2, 1>, chol_reg_smem_bytes(kSolveBounds[5]))) != cudaSuccess) return e;
+  if ((e = gram_set_smem()) != cudaSuccess) return e;
   return adjoint_tc_set_smem();
 }
 
