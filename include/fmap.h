@@ -94,8 +94,8 @@ typedef struct fmap_options {
     int32_t adjoint_kernel;     /* W = Gamma^T C + C^T Gamma, dA_x = Gamma^T A_y - W A_x, dA_y = Gamma A_x,
                                    and the training loss's E = C C^T - I, dL/dC = 4 E C + 2 (C - C_gt):
                                    1 tensor cores (three TF32 passes), 2 CUDA cores (FP32 FMA tiles);
-                                   0 the built-in choice: tensor cores when dA_x has at least two
-                                   128-column tiles per SM, else CUDA cores */
+                                   0 the built-in choice, by the arithmetic of the batch against its
+                                   longest reduction */
     int32_t adjoint_features;   /* tensor-core adjoint GEMMs: output columns per CTA, 64, 128 or 256
                                    (default 128, or 64 below two dA_x tiles per SM) */
     int32_t adjoint_stages;     /* tensor-core adjoint GEMMs: shared-memory stages per CTA, 1 or 2

@@ -1051,7 +1051,7 @@ int32_t adjoint_impl(fmap_batch* b, const float* d_c, const float* a, const floa
   {
     TimedScope ts(b, FMAP_KIND_ADJ_GEMM, st);
     const int ak = b->plan.opt.adjoint_kernel;
-    const bool simt = ak == 2 || (ak == 0 && !b->plan.adj.fills_sms);
+    const bool simt = ak == 2 || (ak == 0 && !b->plan.adj.tensor_cores);
     e = launch_adjoint_gemms(b->dev, b->plan.max_k, b->plan.max_d, a, c, d_mask, d_lambda, b->plan.row_grads, w,
                              simt, st);
     if (e == cudaSuccess && !simt) e = launch_adjoint_tc(b->dev, b->d_adj_items, b->plan.adj, a, c, w, st);
@@ -1177,10 +1177,10 @@ int32_t fmap_loss_orth(fmap_batch* b, const float* c, const float* c_gt, float* 
   cudaError_t e;
   {
     TimedScope ts(b, FMAP_KIND_LOSS, static_cast<cudaStream_t>(stream));
-    // the GEMMs on the tensor cores when the adjoint's run there (both need dL/dC: its tiles
+    // the GEMMs on the tensor cores when the batch is large enough (they need dL/dC: its tiles
     // also carry ||C - C_gt||^2), else the FP32 FMA tiles
     const int ak = b->plan.opt.adjoint_kernel;
-    const bool tc = d_c && !b->plan.loss_tc.items.empty() && (ak == 1 || (ak == 0 && b->plan.adj.fills_sms));
+    const bool tc = d_c && !b->plan.loss_tc.items.empty() && (ak == 1 || (ak == 0 && b->plan.loss_tc.tensor_cores));
     float* w = static_cast<float*>(ws);
     e = tc ? launch_loss_tc(b->dev, b->d_loss_items, b->plan.loss_tc, c, c_gt, loss, d_c, w, w + b->plan.loss_part_off,
                             static_cast<cudaStream_t>(stream))

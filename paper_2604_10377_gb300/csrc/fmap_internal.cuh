@@ -14,8 +14,8 @@
 namespace fmap {
 
 constexpr int kMaxK = 304;
-// per-pair partial sums of the training loss: one per 64 x 64 tile of C
-constexpr int kMaxLossTiles = ((kMaxK + 63) / 64) * ((kMaxK + 63) / 64);
+// per-pair partial sums of the training loss: at most one per 32 x 32 tile of C
+constexpr int kMaxLossTiles = ((kMaxK + 31) / 32) * ((kMaxK + 31) / 32);
 constexpr int kMaxD = 4096;
 // classes of the row solves by k_X (upper bounds): a launch each
 constexpr int kSolveClasses = 6;
@@ -215,7 +215,7 @@ struct AdjTcPlan {
   int n_first = 0;
   int stages = 0;               // shared-memory stages, 1 or 2 (0 on input: the built-in choice)
   int features = 0;             // output columns per CTA, 64, 128 or 256 (0 on input: built-in)
-  bool fills_sms = false;       // at least two dA_x tiles of 128 columns per SM
+  bool tensor_cores = false;    // the batch is large enough for the tensor cores to pay
 };
 // shapes[p] = (k_X, k_Y, d) of pair p; fills the work list, longest reduction first
 void adjoint_tc_plan(const std::vector<int3>& shapes, int sms, AdjTcPlan& P);

@@ -372,6 +372,14 @@ cudaError_t adjoint_tc_set_smem() {
   return set_smem_one<1, kLossNt, true>();
 }
 
+// The tensor cores pay from this many flops of a batch per K-block of its longest chain (the two
+// dependent launches together). A K-block costs them about 4.4 us whatever the batch, the FP32
+// tiles run at 13 to 18 TFLOP/s, the tensor cores at 115 once they fill. Launch times in us, FMA
+// tiles against tensor cores: one pair of k = 200, d = 256 23 / 114, 8 of k = 100, d = 384 27 / 68,
+// 64 of k = 100, d = 256 98 / 78, 16 of k = 200 93 / 121, 32 of k = 200 170 / 139, 128 of k = 30
+// 23 / 35; the loss, 4 of k = 200 27 / 82, 32 of k = 200 94 / 85.
+constexpr double kFlopsPerBlock = 88e6;
+
 void adjoint_tc_plan(const std::vector<int3>& shapes, int sms, AdjTcPlan& P) {
   // shapes[p] = (k_X, k_Y, d) of pair p
   auto build = [&](int nt) {
@@ -395,11 +403,16 @@ void adjoint_tc_plan(const std::vector<int3>& shapes, int sms, AdjTcPlan& P) {
     P.n_first = (int)first.size();
     return (int)second.size();
   };
-  // enough dA_x tiles of 128 columns for two per SM: the tensor cores pay (below that the two
-  // dependent launches are bound by one CTA's reduction loop and the FP32 FMA tiles are faster)
-  P.fills_sms = build(128) >= 2 * sms;
-  if (P.features == 0) P.features = P.fills_sms ? 128 : 64;
+  if (P.features == 0) P.features = build(128) >= 2 * sms ? 128 : 64;
   build(P.features);
+  double flops = 0.0;
+  int blocks = 0;
+  for (const int3& q : shapes) {
+    const double k = q.x, ky = q.y, d = q.z;
+    flops += 4.0 * k * k * ky + 2.0 * ky * k * d + 2.0 * k * (ky + k) * d;
+    blocks = std::max(blocks, (std::max(2 * q.y, q.x) + 31) / 32 + (q.x + q.y + 31) / 32);
+  }
+  P.tensor_cores = flops > kFlopsPerBlock * blocks;
   // one stage: twice the CTAs per SM of two stages, which measured faster at every width
   if (P.stages == 0) P.stages = 1;
 }
@@ -439,6 +452,13 @@ void adjoint_tc_loss_plan(const std::vector<int3>& shapes, AdjTcPlan& P) {
   for (const auto& x : e_items) P.items.push_back(x.second);
   for (const auto& x : g_items) P.items.push_back(x.second);
   P.n_first = (int)e_items.size();
+  double flops = 0.0;
+  int blocks = 0;
+  for (const int3& q : shapes) {
+    flops += 4.0 * q.y * (double)q.y * q.x;
+    blocks = std::max(blocks, (q.x + 31) / 32 + (q.y + 31) / 32);
+  }
+  P.tensor_cores = flops > kFlopsPerBlock * blocks;
   P.features = kLossNt;
   P.stages = 1;
 }
