@@ -80,7 +80,8 @@ typedef struct fmap_options {
     int32_t bwd_group_features; /* tensor-core backward projection: features per CTA group,
                                    64 or 128 (default 128) */
     int32_t bwd_chunk_v;        /* tensor-core backward projection: largest vertex chunk of a work
-                                   item, multiple of 128 in 1024..65536 (default 8192) */
+                                   item, multiple of 128 in 1024..65536 (default 8192; BF16
+                                   features round it up to 256) */
     int32_t solve_threads_k64;  /* row-solve block for k <= 64: 64 or 128 threads (default 64) */
     int32_t solve_threads_k128; /* row-solve block for 64 < k <= 100: 128 or 256 (default 128) */
     /* Persistent CTAs of the tensor-core projections, 1..152 (0 = one per SM, 152). A batch

@@ -98,7 +98,7 @@ struct Plan {
   std::vector<TcBwdItem> bw_items;
   std::vector<int32_t> bw_cta_first;   // bwd_ctas + 1 (FP32) or bwd_ctas / 2 + 1 (BF16) boundaries
   std::vector<TcBwdGroup> bw_groups;
-  int bw_max_img = 0, bw_stages = 0, bw_smem = 0;
+  int bw_max_img = 0, bw_max_nf = 0, bw_stages = 0, bw_smem = 0;
   uint32_t bw_b_bytes = 0;
   // tensor-core adjoint GEMMs (built when the batch is created: the SM count sets the tiles)
   AdjTcPlan adj;
@@ -350,78 +350,76 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
   P.da_int_off = cur;
   cur = align_up(cur + P.a_off[n_shapes], kAlignFloats);
   if (P.tc_bwd) {
-    // Backward work runs on pairs of CTAs (2c, 2c + 1) that walk the same Phi tiles at
-    // the same time, so the second read of each tile hits L2: a shape's features split
-    // into an even number of groups of <= 128, and a work item is (shape, vertex chunk,
-    // pair of groups), one group per CTA of the pair. Items are sorted by cost and dealt
-    // to the CTA pairs round-robin.
+    // Backward work runs on pairs of CTAs (2c, 2c + 1): a work item is (shape, chunk of
+    // 256-vertex tiles, group of <= 256 features, half of them resident in each CTA; the MMA's N
+    // is a multiple of 32). The groups of one chunk follow one another, so that pairs working on
+    // them at the same time share its Phi tiles in L2. Items are sorted by cost and dealt to the
+    // CTA pairs round-robin.
     const int n_ctapairs = P.bwd_ctas / 2;
     int64_t bw_work = 0;
     for (int s = 0; s < n_shapes; ++s)
       if (P.shapes[s].dfeat) bw_work += P.shapes[s].n * (int64_t)((P.shapes[s].d + 255) / 256);
-    const int64_t bw_chunk = opt.bwd_chunk_v ? (int64_t)opt.bwd_chunk_v
-                                             : std::min<int64_t>(kTcChunkV, std::max<int64_t>(
-                                                   1024, (bw_work / (4 * n_ctapairs) + 127) / 128 * 128));
-    const int bw_gf = opt.bwd_group_features ? opt.bwd_group_features : 128;
-    std::vector<TcBwdItem> items;   // pairs: [2 j] for CTA 2c, [2 j + 1] for CTA 2c + 1
+    const int64_t bw_chunk =
+        align_up(opt.bwd_chunk_v ? (int64_t)opt.bwd_chunk_v
+                                 : std::min<int64_t>(kTcChunkV, std::max<int64_t>(1024, bw_work / (4 * n_ctapairs))),
+                 256);
+    const int bw_gf = 2 * (opt.bwd_group_features ? opt.bwd_group_features : 128);
+    std::vector<TcBwdItem> items;
     for (int s = 0; s < n_shapes; ++s) {
       const ShapeDev& sd = P.shapes[s];
       if (!sd.dfeat) continue;
       const int kb = (sd.k + 31) / 32;
-      const int ngroups = 2 * ((sd.d + 2 * bw_gf - 1) / (2 * bw_gf));
-      const int nf_s = ((sd.d + ngroups - 1) / ngroups + 15) / 16 * 16;
+      const int ngroups = (sd.d + bw_gf - 1) / bw_gf;
+      const int nf_s = (int)align_up((sd.d + ngroups - 1) / ngroups, 64);   // whole store boxes but for the last
       std::vector<TcBwdGroup> gl(ngroups);
       for (int g = 0; g < ngroups; ++g) {
         TcBwdGroup& bg = gl[g];
-        bg.shape = s; bg.f0 = g * nf_s; bg.nf = std::max(0, std::min(nf_s, sd.d - bg.f0)); bg.kb = kb;
-        bg.img_off = -1;
-        if (bg.nf <= 0) continue;
+        bg.shape = s; bg.f0 = g * nf_s; bg.nf = (int)align_up(std::min(nf_s, sd.d - bg.f0), 32); bg.kb = kb;
+        if (bg.f0 >= sd.d) { bg.nf = 0; continue; }
         bg.img_off = cur;
         cur = align_up(cur + (int64_t)kb * bg.nf * 32, kAlignFloats);
         P.bw_groups.push_back(bg);
         P.bw_max_img = std::max(P.bw_max_img, kb * bg.nf * 32);
-        P.bw_b_bytes = std::max<uint32_t>(P.bw_b_bytes, (uint32_t)(kb * bg.nf * 128));
+        P.bw_b_bytes = std::max<uint32_t>(P.bw_b_bytes, (uint32_t)(kb * (bg.nf / 2) * 128));
+        P.bw_max_nf = std::max(P.bw_max_nf, bg.nf);
       }
-      for (int gp = 0; gp < ngroups / 2; ++gp)
-        for (int64_t v0 = 0; v0 < sd.n; v0 += bw_chunk)
-          for (int r = 0; r < 2; ++r) {
-            const TcBwdGroup& bg = gl[2 * gp + r];
-            TcBwdItem it{};
-            it.shape = s; it.f0 = bg.f0; it.nf = bg.nf; it.kb = kb;
-            it.v0 = v0; it.v1 = std::min<int64_t>(sd.n, v0 + bw_chunk);
-            it.img_off = bg.img_off;
-            items.push_back(it);
-          }
+      for (int64_t v0 = 0; v0 < sd.n; v0 += bw_chunk)
+        for (const TcBwdGroup& bg : gl) {
+          if (bg.nf == 0) continue;
+          TcBwdItem it{};
+          it.shape = s; it.f0 = bg.f0; it.nf = bg.nf; it.kb = kb;
+          it.v0 = v0; it.v1 = std::min<int64_t>(sd.n, v0 + bw_chunk);
+          it.img_off = bg.img_off;
+          items.push_back(it);
+        }
     }
     if (!items.empty()) {
-      const size_t npi = items.size() / 2;
-      std::vector<int32_t> order(npi);
-      for (size_t i = 0; i < npi; ++i) order[i] = (int32_t)i;
+      std::vector<int32_t> order(items.size());
+      for (size_t i = 0; i < items.size(); ++i) order[i] = (int32_t)i;
       auto bcost = [&](size_t j) {
-        const TcBwdItem& it = items[2 * j];
-        return (double)(it.v1 - it.v0) * (4.0 * P.shapes[it.shape].k + 2.0 * (it.nf + items[2 * j + 1].nf));
+        const TcBwdItem& it = items[j];
+        return (double)(it.v1 - it.v0) * (4.0 * P.shapes[it.shape].k + 2.0 * it.nf);
       };
       std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
         const double cx = bcost(a), cy = bcost(b);
         if (cx != cy) return cx > cy;
         return a < b;
       });
-      // CTA pair c takes pair-items c, c + n_ctapairs, ... of the sorted list, stored contiguously
+      // CTA pair c takes items c, c + n_ctapairs, ... of the sorted list, stored contiguously
       P.bw_cta_first.assign(n_ctapairs + 1, 0);
       for (int c = 0; c < n_ctapairs; ++c) {
-        P.bw_cta_first[c] = (int32_t)(P.bw_items.size() / 2);
-        for (size_t j = c; j < order.size(); j += n_ctapairs) {
-          P.bw_items.push_back(items[2 * order[j]]);
-          P.bw_items.push_back(items[2 * order[j] + 1]);
-        }
+        P.bw_cta_first[c] = (int32_t)P.bw_items.size();
+        for (size_t j = c; j < order.size(); j += n_ctapairs) P.bw_items.push_back(items[order[j]]);
       }
-      P.bw_cta_first[n_ctapairs] = (int32_t)(P.bw_items.size() / 2);
+      P.bw_cta_first[n_ctapairs] = (int32_t)P.bw_items.size();
     }
     const int fixed = 1024 + 512;
     const int out_staging = 8 * 4096;   // BF16 dF staging of the eight epilogue warps
-    P.bw_stages = std::min(6, (kSmemBudget - fixed - out_staging - (int)P.bw_b_bytes) / 16384);
-    if (!P.bw_items.empty() && P.bw_stages < 2) return FMAP_ERR_UNSUPPORTED;
-    P.bw_smem = fixed + out_staging + (int)P.bw_b_bytes + P.bw_stages * 16384;
+    // the operands share what is left: the image of the item in hand, then its Phi stages
+    const int region = (kSmemBudget - fixed - out_staging) / 1024 * 1024;
+    if (!P.bw_items.empty() && (region - (int)P.bw_b_bytes) / 16384 < 2) return FMAP_ERR_UNSUPPORTED;
+    P.bw_b_bytes = (uint32_t)region;
+    P.bw_smem = fixed + out_staging + region;
   }
   if (P.tc_bwd32) {
     // FP32 features: one CTA per SM over (shape, feature group, vertex chunk) items; a
@@ -818,14 +816,15 @@ int32_t fmap_batch_create(fmap_ctx* ctx, const fmap_shape_desc* shapes, int32_t 
         return FMAP_ERR_CUDA;
       }
       put(o_pb + s * (int64_t)sizeof(CUtensorMap), &pb, sizeof(pb));
-      // dF (BF16 or FP32): box 16 features x 32 vertices, stored by the backward projection
+      // FP32 dF: box 32 features x 32 vertices, 128-byte rows with the 128-byte swizzle, stored by the
+      // backward projection
       CUtensorMap dm;
       std::memset(&dm, 0, sizeof(dm));
-      if (sd.dfeat && (P.tc_bwd || P.tc_bwd32)) {
-        cuuint32_t dbox[2] = {16, 32};
-        r = encode(&dm, P.tc_bwd32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, sd.dfeat,
+      if (sd.dfeat && P.tc_bwd32) {
+        cuuint32_t dbox[2] = {32, 32};
+        r = encode(&dm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, sd.dfeat,
                    gdim, gstride, dbox, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) {
           cudaFree(b->dev_mem); delete b;
@@ -1086,7 +1085,10 @@ int32_t project_backward_impl(fmap_batch* b, const float* da, float* w, void* ws
   bp.cta_first = b->d_bw_cta_first;
   bp.stages = P.bw_stages;
   bp.b_bytes_max = P.bw_b_bytes;
-  bp.tmem_cols = P.tc_bwd32 ? 128 : 256;   // two accumulators of <= 64 or <= 128 columns
+  // two accumulators: <= 64 columns each (FP32), or N = bw_max_nf rounded to a power of two
+  bp.tmem_cols = 128;
+  if (!P.tc_bwd32)
+    for (bp.tmem_cols = 64; bp.tmem_cols < 2u * (uint32_t)P.bw_max_nf;) bp.tmem_cols <<= 1;
   bp.ws = w;
   bp.err = static_cast<int*>(ws);
   {

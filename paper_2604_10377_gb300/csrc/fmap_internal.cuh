@@ -133,7 +133,8 @@ struct TcProjParams {
 };
 
 // Work item of the tensor-core backward projection: a vertex chunk of one feature
-// group (nf <= 128 features from f0) of one shape; kb = blocks of 32 basis functions.
+// group (nf features from f0: <= 64, FP32, or a multiple of 32 <= 256, BF16, which may pass d)
+// of one shape; kb = blocks of 32 basis functions.
 struct TcBwdItem {
   int32_t shape, f0, nf, kb;
   int64_t v0, v1;
@@ -148,13 +149,12 @@ struct TcBwdGroup {
 struct TcBwdParams {
   const ShapeDev* shapes;
   const CUtensorMap* phimaps;  // per shape: FP32 Phi, box 32 x 64, 128-byte swizzle
-  const CUtensorMap* dfmaps;   // per shape: dF (BF16 or FP32), box 16 x 32, no swizzle (TMA stores)
-  const TcBwdItem* items;       // BF16: item j of CTA pair c is [2 j] for CTA 2c, [2 j + 1] for CTA 2c + 1;
-                                //   FP32: one item per entry
+  const CUtensorMap* dfmaps;   // FP32, per shape: dF, box 32 features x 32 vertices, 128-byte swizzle (TMA stores)
+  const TcBwdItem* items;
   const int32_t* cta_first;     // BF16: CTA pair c owns items [cta_first[c], cta_first[c + 1]);
                                 //   FP32: CTA c
-  int32_t stages;
-  uint32_t b_bytes_max;
+  int32_t stages;               // FP32: Phi stages
+  uint32_t b_bytes_max;         // FP32: bytes of the largest image; BF16: of the operands' region
   uint32_t tmem_cols;
   const float* ws;
   int* err;

@@ -30,8 +30,7 @@ constexpr int kConvWarps = 4;
 constexpr int kThreads = 32 * (2 + kEpiWarps + kConvWarps);
 constexpr int kTileV = 128;                          // vertices per output tile (MMA M)
 constexpr uint32_t kAStageBytes = kTileV * 128;      // 128 rows x 32 FP32
-constexpr uint32_t kOutChunkBytes = 32 * 16 * 4;     // 32 rows x 16 FP32: one TMA store box
-constexpr uint32_t kOutWarpBytes = 2 * kOutChunkBytes;   // <= 32 features per warp and tile
+constexpr uint32_t kOutWarpBytes = 32 * 128;         // 32 rows x 32 FP32: one TMA store box per epilogue warp
 
 // x minus the TF32 value the tensor core reads for it (the low 13 bits dropped): exact.
 __device__ __forceinline__ float tf32_trunc_rest(float x) {
@@ -210,27 +209,34 @@ __global__ void __launch_bounds__(kThreads, 1) project_bwd_tc32_kernel(TcBwdPara
         const float m = v < item.v1 ? __ldg(s.mass + v) : 0.f;
         if (!tc::mbar_wait(&acc_full[buf], acc_phase[buf], abort_flag)) goto epi_done;
         tc::tc_fence_after();
-        if (lane == 0) tc::bulk_wait_group_read0();
-        __syncwarp();
-        int j = 0;
-        for (int ch = half; ch < item.nf / 16; ch += 2, ++j) {
-          float x[16];
-          tc::tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * (P.tmem_cols / 2) + ch * 16),
-                        x);
-          float4* dst = reinterpret_cast<float4*>(stage_out + j * kOutChunkBytes + lane * 64);
+        // 32 features per warp, 128-byte rows with the 128-byte swizzle (conflict-free, and half as
+        // many box rows as 16 features would make: a TMA store takes about 6 cycles per row)
+        const int c0 = 32 * half, nv = item.nf - c0;
+        float x[32];
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            dst[q] = make_float4(x[4 * q] * m, x[4 * q + 1] * m, x[4 * q + 2] * m, x[4 * q + 3] * m);
-        }
+        for (int q = 0; q < 2; ++q)
+          if (16 * q < nv)
+            tc::tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) +
+                              (uint32_t)(buf * (P.tmem_cols / 2) + c0 + 16 * q),
+                          *reinterpret_cast<float(*)[16]>(x + 16 * q));
         tc::tc_fence_before();
-        tc::fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&acc_empty[buf]);
-        if (lane == 0 && vrow0 < s.n) {
-          j = 0;
-          for (int ch = half; ch < item.nf / 16; ch += 2, ++j)
-            tc::tma_store_2d(dmap, stage_out + j * kOutChunkBytes, item.f0 + ch * 16, (int)vrow0);
-          tc::bulk_commit_group();
+        if (lane == 0) {
+          tc::mbar_arrive(&acc_empty[buf]);
+          tc::bulk_wait_group_read0();     // the previous box's store has read the buffer
+        }
+        __syncwarp();
+        if (nv > 0 && vrow0 < s.n) {
+#pragma unroll
+          for (int z = 0; z < 8; ++z)
+            *reinterpret_cast<float4*>(stage_out + lane * 128 + ((z ^ (lane & 7)) << 4)) =
+                make_float4(x[4 * z] * m, x[4 * z + 1] * m, x[4 * z + 2] * m, x[4 * z + 3] * m);
+          tc::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tc::tma_store_2d(dmap, stage_out, item.f0 + c0, (int)vrow0);
+            tc::bulk_commit_group();
+          }
         }
         acc_phase[buf] ^= 1;
         buf ^= 1;
