@@ -92,6 +92,7 @@ struct Plan {
   std::vector<int32_t> tc_cta_first;   // proj_ctas + 1 entries per launch
   std::vector<TcLaunch> tc_launches;
   std::vector<TcRedGroup> tc_groups;
+  std::vector<int64_t> tc_parts;       // offsets of the partials, group after group
   int64_t tc_max_group_elems = 0;
   int tc_smem = 0;                     // the largest dynamic shared memory of the launches
   // tensor-core backward projection
@@ -264,7 +265,7 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
         const uint32_t pb = P.tc32 ? kbu * 4096u + (uint32_t)u.npad * 256u
                                    : std::max<uint32_t>(kbu * 8192u, (uint32_t)u.npad * 256u);
         pmax = std::max<uint32_t>(pmax, pb);
-        tmax = std::max<uint32_t>(tmax, (uint32_t)(u.fg * u.npad));
+        tmax = std::max<uint32_t>(tmax, (uint32_t)(u.fg * u.npad) * (!P.tc32 && tc_merged(u.fg, u.npad) ? 2u : 1u));
       }
       TcLaunch L{};
       L.cta_off = (int32_t)P.tc_cta_first.size();
@@ -280,7 +281,7 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
         TcRedGroup rg{};
         rg.shape = u.s; rg.f0 = u.f0; rg.stride = u.fg * 128; rg.dspan = u.dspan;
         rg.n0 = u.n0; rg.nk = u.nk;
-        rg.it_beg = (int32_t)P.tc_items.size();
+        rg.part_beg = (int32_t)P.tc_parts.size();
         int64_t v = 0;
         while (v < sd.n) {
           int64_t take = (int64_t)std::ceil(std::max(budget, 0.0) / u.cpv);
@@ -296,6 +297,7 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
           it.part_off = cur;
           cur = align_up(cur + (int64_t)u.nk * rg.stride, kAlignFloats);
           P.tc_items.push_back(it);
+          P.tc_parts.push_back(it.part_off);
           v += take;
           budget -= u.cpv * (double)take;
           if (budget <= 1e-9 * per_cta && cta < nctas - 1) {
@@ -304,7 +306,7 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
             budget += per_cta;
           }
         }
-        rg.it_end = (int32_t)P.tc_items.size();
+        rg.part_end = (int32_t)P.tc_parts.size();
         P.tc_groups.push_back(rg);
         P.tc_max_group_elems = std::max<int64_t>(P.tc_max_group_elems, (int64_t)u.nk * rg.dspan);
       }
@@ -566,6 +568,7 @@ struct fmap_batch {
   const TcItem* d_tc_items = nullptr;
   const int32_t* d_tc_cta_first = nullptr;
   const TcRedGroup* d_tc_groups = nullptr;
+  const int64_t* d_tc_parts = nullptr;
   const CUtensorMap* d_phimaps_fwd = nullptr;
   const CUtensorMap* d_massmaps = nullptr;
   const CUtensorMap* d_dfmaps = nullptr;
@@ -729,7 +732,8 @@ int32_t fmap_batch_create(fmap_ctx* ctx, const fmap_shape_desc* shapes, int32_t 
   const int64_t o_ti = o_tm + bytes_of(P.shapes.size(), sizeof(CUtensorMap));
   const int64_t o_to = o_ti + bytes_of(P.tc_items.size(), sizeof(TcItem));
   const int64_t o_tg = o_to + bytes_of(P.tc_cta_first.size(), sizeof(int32_t));
-  const int64_t o_fp = o_tg + bytes_of(P.tc_groups.size(), sizeof(TcRedGroup));
+  const int64_t o_tp = o_tg + bytes_of(P.tc_groups.size(), sizeof(TcRedGroup));
+  const int64_t o_fp = o_tp + bytes_of(P.tc_parts.size(), sizeof(int64_t));
   const int64_t o_mm = o_fp + bytes_of(P.shapes.size(), sizeof(CUtensorMap));
   const int64_t o_dm = o_mm + bytes_of(P.shapes.size(), sizeof(CUtensorMap));
   const int64_t o_pb = o_dm + bytes_of(P.shapes.size(), sizeof(CUtensorMap));
@@ -844,6 +848,7 @@ int32_t fmap_batch_create(fmap_ctx* ctx, const fmap_shape_desc* shapes, int32_t 
     put(o_ti, P.tc_items.data(), P.tc_items.size() * sizeof(TcItem));
     put(o_to, P.tc_cta_first.data(), P.tc_cta_first.size() * sizeof(int32_t));
     put(o_tg, P.tc_groups.data(), P.tc_groups.size() * sizeof(TcRedGroup));
+    put(o_tp, P.tc_parts.data(), P.tc_parts.size() * sizeof(int64_t));
     e = P.tc32 ? project_tc32_set_smem(P.tc_smem) : project_tc_set_smem(P.tc_smem);
     if (e != cudaSuccess) { cudaFree(b->dev_mem); delete b; return cuda_fail(e, "cudaFuncSetAttribute(project)"); }
   }
@@ -862,6 +867,7 @@ int32_t fmap_batch_create(fmap_ctx* ctx, const fmap_shape_desc* shapes, int32_t 
   b->d_tc_items = reinterpret_cast<const TcItem*>(base + o_ti);
   b->d_tc_cta_first = reinterpret_cast<const int32_t*>(base + o_to);
   b->d_tc_groups = reinterpret_cast<const TcRedGroup*>(base + o_tg);
+  b->d_tc_parts = reinterpret_cast<const int64_t*>(base + o_tp);
   b->d_phimaps_fwd = reinterpret_cast<const CUtensorMap*>(base + o_fp);
   b->d_massmaps = reinterpret_cast<const CUtensorMap*>(base + o_mm);
   b->d_dfmaps = reinterpret_cast<const CUtensorMap*>(base + o_dm);
@@ -965,7 +971,7 @@ int32_t fmap_project(fmap_batch* b, float* a_out, void* ws, size_t ws_bytes, voi
   }
   {
     TimedScope ts(b, FMAP_KIND_PROJECT_REDUCE, st);
-    e = launch_project_tc_reduce(b->dev.shapes, b->d_tc_items, b->d_tc_groups, (int)P.tc_groups.size(),
+    e = launch_project_tc_reduce(b->dev.shapes, b->d_tc_parts, b->d_tc_groups, (int)P.tc_groups.size(),
                                  P.tc_max_group_elems, a_out, w, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "project_reduce");

@@ -108,13 +108,17 @@ struct TcItem {
   int64_t part_off;    // float offset (workspace) of the segment's partial, nk x (fg*128)
 };
 
-// Items [it_beg, it_end) hold the partials of basis rows n0 .. n0+nk and features
-// f0 .. f0+dspan of one shape.
+// Entries [part_beg, part_end) of the list of partials (float offsets in the workspace) hold the
+// partials of basis rows n0 .. n0+nk and features f0 .. f0+dspan of one shape.
 struct TcRedGroup {
   int32_t shape, f0, dspan, stride;
   int32_t n0, nk;
-  int32_t it_beg, it_end;
+  int32_t part_beg, part_end;
 };
+
+// BF16 features: whether an item's hi and lo products run as one MMA of N = 2 npad columns per
+// feature group (N at most 256, the accumulators in 512 TMEM columns).
+__host__ __device__ __forceinline__ bool tc_merged(int fg, int npad) { return npad <= 128 && 2 * fg * npad <= 512; }
 
 struct TcProjParams {
   const ShapeDev* shapes;
@@ -174,7 +178,7 @@ cudaError_t project_tc32_set_smem(int bytes);
 cudaError_t launch_project_tc32(const TcProjParams& p, int grid, int smem_bytes, cudaStream_t st);
 int project_tc_threads();
 cudaError_t launch_project_tc(const TcProjParams& p, int grid, int smem_bytes, cudaStream_t st);
-cudaError_t launch_project_tc_reduce(const ShapeDev* shapes, const TcItem* items, const TcRedGroup* groups,
+cudaError_t launch_project_tc_reduce(const ShapeDev* shapes, const int64_t* parts, const TcRedGroup* groups,
                                      int n_groups, int64_t max_elems, float* a_out, const float* ws,
                                      cudaStream_t st);
 

@@ -12,8 +12,12 @@
 //               split it into BF16 hi + lo (P = hi + lo to ~2^-17), written in place
 //               over the Phi tile as K-major 128-byte-swizzled B tiles: the mass is
 //               fused into the operand load;
-//   warp 1      issues tcgen05.mma (M = 128 features, N = k rounded up to 16,
-//               K = 16 vertices) for hi and lo into FP32 accumulators in TMEM.
+//   warp 1      issues tcgen05.mma (M = 128 features, K = 16 vertices) into FP32 accumulators
+//               in TMEM: N = k rounded up to 16 for hi and for lo, or, where the columns
+//               allow it (tc_merged), one MMA on the rows of hi and lo together, whose two
+//               accumulators the epilogue adds. An MMA of small N is bound by its reads of the F
+//               tile, which two MMAs take twice: 64 shapes of n = 50000, d = 256 at k = 30 /
+//               50 / 100 took 433 / 454 / 500 us with two and 380 / 405 / 470 with one.
 // At the end of a segment warps 2-9 read the accumulators back (tcgen05.ld) and
 // write the segment's partial A; a second kernel adds the partials of each shape
 // in a fixed order. F is exact in BF16, so A carries only the ~2^-17 error of
@@ -126,7 +130,9 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
         const TcItem item = P.items[it];
         if (!tc::mbar_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
         tc::tc_fence_after();
-        const uint32_t idesc = tc::idesc_bf16_f32(128, (uint32_t)item.npad, 1, 0);
+        const bool merged = tc_merged(item.fg, item.npad);
+        const uint32_t cols = (uint32_t)item.npad * (merged ? 2u : 1u);      // accumulator columns per feature group
+        const uint32_t idesc = tc::idesc_bf16_f32(128, cols, 1, 0);
         const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
         bool ok = true;
         for (int st = 0; st < nst && ok; ++st) {
@@ -143,9 +149,9 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
             for (int m = 0; m < item.fg; ++m) {
               const uint64_t ad = tc::smem_desc(a_base + m * 2 * kBoxBytes + kk * 2048, kBoxBytes, 1024,
                                                 tc::kLayoutSW128);
-              const uint32_t d = tmem_base + (uint32_t)(m * item.npad);
+              const uint32_t d = tmem_base + (uint32_t)m * cols;
               tc::mma_bf16(d, ad, bh, idesc, (st | kk) != 0 ? 1u : 0u);
-              tc::mma_bf16(d, ad, bl, idesc, 1u);
+              if (!merged) tc::mma_bf16(d, ad, bl, idesc, 1u);
             }
           }
           tc::mma_commit(&empty[stage]);
@@ -234,12 +240,20 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
         const int quarter = warp & 3, half = cw >> 2;
         const int stride = item.fg * 128;
         float* part = P.ws + item.part_off;
+        const bool merged = tc_merged(item.fg, item.npad);
+        const int cols = item.npad * (merged ? 2 : 1);
         for (int m = 0; m < item.fg; ++m) {
           const int fl = m * 128 + quarter * 32 + lane;
           const bool fok = item.f0 + fl < s.d;
           for (int ch = half; ch < item.npad / 16; ch += 2) {
             float v[16];
-            tc::tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(m * item.npad + ch * 16), v);
+            tc::tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(m * cols + ch * 16), v);
+            if (merged) {
+              float w[16];
+              tc::tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(m * cols + item.npad + ch * 16), w);
+#pragma unroll
+              for (int t = 0; t < 16; ++t) v[t] += w[t];
+            }
             if (fok) {
 #pragma unroll
               for (int t = 0; t < 16; ++t) {
@@ -263,27 +277,51 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
   if (threadIdx.x == 0 && *abort_flag) atomicExch(P.err, (int)FMAP_ERR_TIMEOUT);
 }
 
-// A_s[n0 + n][f0 + f] = sum over the group's items (in order) of partial[n][f].
-__global__ void project_tc_reduce_kernel(const ShapeDev* shapes, const TcItem* items, const TcRedGroup* groups,
-                                         float* a_out, const float* ws) {
+// A_s[n0 + n][f0 + f] = sum over the group's partials [n][f], in a fixed order: four thread groups
+// take every fourth partial, four loads in flight each, and their sums are added in order (one
+// thread adding every partial waits for one L2 round trip after another: one pair of n = 5000,
+// 76 partials per shape: 17 us against 11).
+__global__ void __launch_bounds__(256) project_tc_reduce_kernel(const ShapeDev* shapes, const int64_t* parts,
+                                                                const TcRedGroup* groups, float* a_out, const float* ws) {
+  __shared__ float4 red[3][64];
   const TcRedGroup g = groups[blockIdx.y];
   const ShapeDev s = shapes[g.shape];
   // four consecutive features per thread (dspan, f0, d are multiples of 16 and the
   // partials are 256-byte aligned; float4 stores when the output buffer is 16-byte aligned)
   const int q4 = g.dspan >> 2, total = g.nk * q4;
   const bool vec = (reinterpret_cast<uintptr_t>(a_out) & 15) == 0;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+  const int sub = threadIdx.x >> 6, lane = threadIdx.x & 63;
+  for (int e0 = blockIdx.x * 64; e0 < total; e0 += gridDim.x * 64) {
+    const int e = e0 + lane;
     const int n = e / q4, f = (e - n * q4) * 4;
+    const float* src = ws + (int64_t)n * g.stride + f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = g.it_beg; i < g.it_end; ++i) {
-      const float4 u = *reinterpret_cast<const float4*>(ws + items[i].part_off + (int64_t)n * g.stride + f);
-      acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
+    if (e < total) {
+      for (int i = g.part_beg + sub; i < g.part_end; i += 16) {
+        float4 u[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          u[j] = i + 4 * j < g.part_end ? *reinterpret_cast<const float4*>(src + __ldg(parts + i + 4 * j))
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { acc.x += u[j].x; acc.y += u[j].y; acc.z += u[j].z; acc.w += u[j].w; }
+      }
     }
-    float* o = a_out + s.a_off + (int64_t)(g.n0 + n) * s.d + g.f0 + f;
-    if (vec) {
-      *reinterpret_cast<float4*>(o) = acc;
-    } else {
-      o[0] = acc.x; o[1] = acc.y; o[2] = acc.z; o[3] = acc.w;
+    __syncthreads();                   // (the previous round's sums have been read)
+    if (sub > 0) red[sub - 1][lane] = acc;
+    __syncthreads();
+    if (sub == 0 && e < total) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const float4 u = red[j][lane];
+        acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
+      }
+      float* o = a_out + s.a_off + (int64_t)(g.n0 + n) * s.d + g.f0 + f;
+      if (vec) {
+        *reinterpret_cast<float4*>(o) = acc;
+      } else {
+        o[0] = acc.x; o[1] = acc.y; o[2] = acc.z; o[3] = acc.w;
+      }
     }
   }
 }
@@ -302,12 +340,12 @@ cudaError_t launch_project_tc(const TcProjParams& p, int grid, int smem_bytes, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_project_tc_reduce(const ShapeDev* shapes, const TcItem* items, const TcRedGroup* groups,
+cudaError_t launch_project_tc_reduce(const ShapeDev* shapes, const int64_t* parts, const TcRedGroup* groups,
                                      int n_groups, int64_t max_elems, float* a_out, const float* ws,
                                      cudaStream_t st) {
   if (n_groups <= 0) return cudaSuccess;
-  dim3 grid((unsigned)std::min<int64_t>((max_elems / 4 + 255) / 256, 4096), (unsigned)n_groups);
-  project_tc_reduce_kernel<<<grid, 256, 0, st>>>(shapes, items, groups, a_out, ws);
+  dim3 grid((unsigned)std::min<int64_t>((max_elems / 4 + 63) / 64, 4096), (unsigned)n_groups);
+  project_tc_reduce_kernel<<<grid, 256, 0, st>>>(shapes, parts, groups, a_out, ws);
   return cudaGetLastError();
 }
 
