@@ -29,7 +29,8 @@ constexpr int64_t kTcChunkV = 8192;    // vertices per work item of the tensor-c
 constexpr int kTcCtas = 152;           // persistent CTAs of the projection (one per GB300 SM)
 constexpr int64_t kStageV = 64;        // vertices per projection pipeline stage
 constexpr int64_t kTcSegMaxV = 8192;   // longest projection segment (one TMEM accumulation), BF16 F
-constexpr int64_t kTc32SegMaxV = 512;   // the same for FP32 F (accuracy of the TF32 passes)
+constexpr int64_t kTc32SegMaxV[3] = {512, 2048, 2048};   // the same for FP32 F, by its accumulators
+constexpr int64_t kTc32StageV = 32;    // vertices per stage, FP32 F
 constexpr int kSmemBudget = 227 * 1024;
 
 int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
@@ -67,7 +68,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 struct TcLaunch {
   int32_t cta_off;     // offset of its proj_ctas + 1 CTA boundaries in tc_cta_first
   int32_t stages;
-  uint32_t f_stage, p_stage, tmem_cols;
+  uint32_t f_stage, p_stage, part, tmem_cols;
   int32_t smem;
 };
 
@@ -208,16 +209,17 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
     // class a stream-K split of the vertex ranges into proj_ctas ranges of equal cost
     // (64-vertex granularity)
     // A spectral size above the widest basis range of one unit (256, the MMA's largest
-    // N, for BF16 features; 128 for FP32 features, whose stages are larger) is split
-    // into basis ranges of equal width (a multiple of 32), each reading its own Phi
-    // columns and all of F.
+    // N, for BF16 features; 208 for FP32 features, two feature groups of which share 512
+    // TMEM columns with their operand slots) is split into basis ranges of equal width (a
+    // multiple of 32; of 16 for FP32), each reading its own Phi columns and all of F.
     struct Unit { int s, f0, fg, npad, n0, nk, dspan; double cpv; };
     std::vector<Unit> classes[4];
-    const int nmax = P.tc32 ? 128 : 256;
+    const int nmax = P.tc32 ? 208 : 256;
+    const int nround = P.tc32 ? 16 : 32;
     for (int s = 0; s < n_shapes; ++s) {
       const ShapeDev& sd = P.shapes[s];
       const int nsplit = (sd.k + nmax - 1) / nmax;
-      const int width = ((sd.k + nsplit - 1) / nsplit + 31) / 32 * 32;
+      const int width = ((sd.k + nsplit - 1) / nsplit + nround - 1) / nround * nround;
       for (int h = 0; h < nsplit; ++h) {
         const int n0 = h * width;
         const int nk = std::min(width, sd.k - n0);
@@ -225,12 +227,7 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
         const int npad = (nk + 15) / 16 * 16;
         const int mt = (sd.d + 127) / 128;
         int fg_cap = std::max(1, std::min(4, 512 / npad));
-        if (P.tc32) {
-          // two stages of (F + its remainder: 32 KB per group) + Phi, Ph, Pl must fit
-          const int pb = (npad + 31) / 32 * 4096 + npad * 256;
-          fg_cap = std::max(1, std::min(std::min(fg_cap, 2), ((kSmemBudget - 1536) / 2 - pb - 128) / 32768));
-          fg_cap = std::max(1, std::min(fg_cap, 256 / npad));   // two accumulators in 512 TMEM columns
-        }
+        if (P.tc32) fg_cap = std::min(2, 512 / (npad + kTc32Slots * kTc32SlotCols));
         const int groups = (mt + fg_cap - 1) / fg_cap;
         const int fg_s = (mt + groups - 1) / groups;
         const int cls = npad <= 32 ? 0 : (npad <= 64 ? 1 : (npad <= 128 ? 2 : 3));
@@ -244,28 +241,28 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
         }
       }
     }
-    // The tensor cores accumulate a segment in TMEM; the FP32-feature kernel bounds that
-    // chain to 512 vertices (64 K-steps) so that the accumulator's rounding stays in the
-    // FP32 class (a longer chain drifts, ~6e-8 relative per K-step); partials are then
-    // added in IEEE FP32 by the reduction. The tuning knob applies to BF16 features.
-    const int64_t seg_max = P.tc32 ? kTc32SegMaxV : (opt.proj_seg_max_v ? (int64_t)opt.proj_seg_max_v : kTcSegMaxV);
+    // The tensor cores accumulate a segment in TMEM, and the chain's rounding grows with its
+    // adds (~6e-8 relative each); partials are then added in IEEE FP32 by the reduction. The
+    // FP32-feature kernel keeps the chain in the FP32 class: 2048 vertices (128 adds) where the
+    // heads' products have an accumulator of their own, 512 (192 adds) where they share it.
+    // The tuning knob applies to BF16 features.
     // vertices per pipeline stage: 64 (BF16 F, one 128-byte row of BF16) or 32 (FP32 F)
-    const int64_t stage_v = P.tc32 ? 32 : kStageV;
+    const int64_t stage_v = P.tc32 ? kTc32StageV : kStageV;
     for (int cls = 0; cls < 4; ++cls) {
       const std::vector<Unit>& units = classes[cls];
       if (units.empty()) continue;
-      uint32_t fmax = 0, pmax = 0, tmax = 0;
+      uint32_t fmax = 0, pmax = 0, tmax = 0, part = 0;
       double total = 0.0;
       for (const Unit& u : units) {
         total += u.cpv * (double)P.shapes[u.s].n;
         // BF16: F tile; Phi tile converted in place into P hi / lo.
-        // FP32: F tile and its TF32 remainder; Phi tile, then P hi and P lo beside it.
+        // FP32: F and Phi tiles of 32 vertices; the basis parts have slots of their own.
         const uint32_t kbu = (uint32_t)((u.npad + 31) / 32);
-        fmax = std::max<uint32_t>(fmax, (uint32_t)u.fg * (P.tc32 ? 32768u : 16384u));
-        const uint32_t pb = P.tc32 ? kbu * 4096u + (uint32_t)u.npad * 256u
-                                   : std::max<uint32_t>(kbu * 8192u, (uint32_t)u.npad * 256u);
+        fmax = std::max<uint32_t>(fmax, (uint32_t)u.fg * 16384u);
+        const uint32_t pb = P.tc32 ? kbu * 4096u : std::max<uint32_t>(kbu * 8192u, (uint32_t)u.npad * 256u);
         pmax = std::max<uint32_t>(pmax, pb);
-        tmax = std::max<uint32_t>(tmax, (uint32_t)(u.fg * u.npad) * (!P.tc32 && tc_merged(u.fg, u.npad) ? 2u : 1u));
+        if (P.tc32) part = std::max<uint32_t>(part, 3u * (uint32_t)((u.npad + 63) / 64) * 2048u);
+        tmax = std::max<uint32_t>(tmax, (uint32_t)(u.fg * u.npad) * (tc_merged(u.fg, u.npad) ? 2u : 1u));
       }
       TcLaunch L{};
       L.cta_off = (int32_t)P.tc_cta_first.size();
@@ -282,6 +279,8 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
         rg.shape = u.s; rg.f0 = u.f0; rg.stride = u.fg * 128; rg.dspan = u.dspan;
         rg.n0 = u.n0; rg.nk = u.nk;
         rg.part_beg = (int32_t)P.tc_parts.size();
+        const int64_t seg_max = P.tc32 ? kTc32SegMaxV[tc32_accs(u.fg, u.npad) - 1]
+                                       : (opt.proj_seg_max_v ? (int64_t)opt.proj_seg_max_v : kTcSegMaxV);
         int64_t v = 0;
         while (v < sd.n) {
           int64_t take = (int64_t)std::ceil(std::max(budget, 0.0) / u.cpv);
@@ -311,13 +310,14 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
         P.tc_max_group_elems = std::max<int64_t>(P.tc_max_group_elems, (int64_t)u.nk * rg.dspan);
       }
       for (int c = cta + 1; c <= nctas; ++c) first[c] = (int32_t)P.tc_items.size();
-      L.f_stage = std::max<uint32_t>(fmax, 16384u);
-      L.p_stage = (std::max<uint32_t>(pmax, 8192u) + 1023u) / 1024u * 1024u;
-      uint32_t cols = 32;
-      while (cols < (P.tc32 ? 2 * tmax : tmax)) cols <<= 1;   // FP32: two accumulators
+      L.f_stage = P.tc32 ? fmax : std::max<uint32_t>(fmax, 16384u);
+      L.p_stage = P.tc32 ? pmax : (std::max<uint32_t>(pmax, 8192u) + 1023u) / 1024u * 1024u;
+      L.part = part;
+      uint32_t cols = P.tc32 ? 512 : 32;   // FP32: accumulators and operand slots
+      while (cols < tmax) cols <<= 1;
       L.tmem_cols = cols;
-      const int fixed = 1024 + 512;
-      const int per_stage = (int)(L.f_stage + L.p_stage) + (int)stage_v * 4;
+      const int fixed = 1024 + 512 + (P.tc32 ? kTc32Slots * (int)part : 0);
+      const int per_stage = (int)(L.f_stage + L.p_stage) + (int)stage_v * 4;   // (masses: a multiple of 128 bytes)
       L.stages = std::min(opt.proj_max_stages ? opt.proj_max_stages : 6, (kSmemBudget - fixed) / per_stage);
       if (L.stages < 2) return FMAP_ERR_UNSUPPORTED;
       L.smem = fixed + L.stages * per_stage;
@@ -960,6 +960,7 @@ int32_t fmap_project(fmap_batch* b, float* a_out, void* ws, size_t ws_bytes, voi
     tp.stages = L.stages;
     tp.f_stage_bytes = L.f_stage;
     tp.p_stage_bytes = L.p_stage;
+    tp.part_bytes = L.part;
     tp.tmem_cols = L.tmem_cols;
     tp.ws = w;
     tp.err = static_cast<int*>(ws);

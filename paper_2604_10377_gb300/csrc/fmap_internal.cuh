@@ -131,10 +131,20 @@ struct TcProjParams {
   int32_t stages;
   uint32_t f_stage_bytes;
   uint32_t p_stage_bytes;
+  uint32_t part_bytes;        // FP32 features: one slot of the basis parts
   uint32_t tmem_cols;
   float* ws;
   int* err;                   // workspace error word
 };
+
+// FP32 features: operand slots and TMEM columns of one slot per feature group (three BF16 parts of 16
+// vertices). Accumulators per feature group that fit beside the slots: three, one MMA per third of F
+// on all thirds of P that it meets (N at most 256); two, the heads' products apart from the rest; one.
+constexpr int kTc32Slots = 2, kTc32SlotCols = 24;
+__host__ __device__ __forceinline__ int tc32_accs(int fg, int npad) {
+  if (3 * npad <= 256 && fg * (3 * npad + kTc32Slots * kTc32SlotCols) <= 512) return 3;
+  return fg * (2 * npad + kTc32Slots * kTc32SlotCols) <= 512 ? 2 : 1;
+}
 
 // Work item of the tensor-core backward projection: a vertex chunk of one feature
 // group (nf features from f0: <= 64, FP32, or a multiple of 32 <= 256, BF16, which may pass d)

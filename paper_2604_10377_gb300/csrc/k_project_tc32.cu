@@ -1,70 +1,145 @@
-// Spectral projection on the tensor cores (Eq. 1) for FP32 features, three-pass TF32:
+// Spectral projection on the tensor cores (Eq. 1) for FP32 features, by BF16 thirds:
 //
 //   A_s^T (d x k) = F_s^T (d x n) . P_s (n x k),   P_s = diag(M_s) Phi_s
 //
-// TF32 keeps 10 explicit mantissa bits of each operand; a single pass would leave
-// ~2^-11 relative error per product. Each operand is therefore split into a TF32 head
-// (rounded to nearest) and the exact FP32 remainder, P = Ph + Pl and F = Fh + Fl, and
-// three products are accumulated in FP32:
-//   Ph.Fh + Pl.Fh + Ph.Fl,
-// which drops Pl.Fl (~2^-22) and the TF32 truncation of the two correction terms
-// (~2^-21 each): the accuracy class of an FP32 accumulation.
+// Each FP32 operand is the exact sum of three BF16 numbers (head, middle, tail: 8 bits each,
+// rounded to nearest), F = Fh + Fm + Fl and P = Ph + Pm + Pl. Six of the nine products are
+// accumulated in FP32,
+//   Fh.Ph + (Fh.Pm + Fm.Ph) + (Fh.Pl + Fm.Pm + Fl.Ph),
+// which leaves out less than 2^-26 of a product: nothing that FP32 accumulation keeps.
+//
+// What bounds it: at small k the reads of F and Phi, and beside them what a stage costs each
+// role in turn (issuing its copies and MMAs, splitting, handing over); from k ~ 100 the MMAs and
+// the partials. An operand that a converter writes to shared memory costs its write and one read
+// per MMA, so the thirds of F go to TMEM (the A operand of the MMA may come from there; a thread
+// holds one feature, whose vertices are the K dimension, and no transpose is left), and only the
+// thirds of P, the smaller operand, are written to shared memory, in vertex rows as they arrive.
+// 32 shapes of n = 50000, d = 256 (3.0 GB at k = 200), against two TF32 parts of each operand in
+// shared memory, F transposed, three MMAs: k = 30 646 -> 356 us, k = 50 702 -> 360 us, k = 100
+// 809 -> 513 us, k = 200 (two passes over F then, one now) 1718 -> 701 us; error against 64 bits
+// at k = 50 3.3e-6 -> 7e-7, at k = 200 3.5e-6 -> 3.2e-6. One lane issuing all copies of a
+// stage: 420 us at k = 50; MMA descriptors built between the MMAs: 422 us; twice the converter
+// warps: 371 us; three or four slots: no gain; stages of one step: 600 us.
 //
 // Same schedule as the BF16 kernel (one persistent CTA per SM over a stream-K range of
-// (shape, feature group) segments, partials reduced in a fixed order by a second
-// kernel), with 32-vertex stages and two TMEM accumulators (segments are short, so the
-// epilogue of one overlaps the MMAs of the next):
-//   warp 0      TMA-loads the F tile (FP32, MN-major: 32-feature boxes, 128-byte
-//               swizzle), the Phi tile (FP32, 32-column boxes) and the 32 masses;
-//   warps 2-9   form P = M * Phi and write Ph, Pl as K-major 128-byte-swizzled B tiles
-//               (the mass is fused into the operand load), and transpose the F tile into
-//               K-major A tiles Fh (in place) and Fl (kind::tf32 takes K-major operands
-//               only);
-//   warp 1      issues tcgen05.mma kind::tf32 (M = 128 features, N = k rounded up to 16,
-//               K = 8 vertices), three per K-step, into FP32 accumulators in TMEM.
-// Waits are bounded like the BF16 kernel's.
+// (shape, feature group) segments, partials reduced in a fixed order by a second kernel), with
+// stages of 32 vertices (two K-steps of 16):
+//   warp 0       TMA-loads the F tile (FP32, 32-feature boxes, 128-byte swizzle), the Phi tile
+//                (FP32, 32-column boxes) and the masses;
+//   warps 2-9    read one feature per lane, split it and store the thirds to a slot of TMEM;
+//   warps 10-13  form P = M * Phi, split it and write the thirds to a slot of shared memory
+//                (B operand, MN-major, 128-byte swizzle, 64 columns per group);
+//   warp 1       issues tcgen05.mma kind::f16 (M = 128 features, N = k rounded up to 16, K = 16
+//                vertices): six per feature group and step, or three, one per third of F on all
+//                thirds of P that it meets, where three accumulators fit (tc32_accs). With an
+//                accumulator of its own the heads' chain has one add per step, and the rounding
+//                of the others is 2^-8 smaller.
+// Warps 2-9 write a segment's partial at its end. Waits are bounded like the BF16 kernel's.
 #include "fmap_internal.cuh"
 #include "tc_ptx.cuh"
 
 namespace fmap {
 namespace {
 
-constexpr int kConvWarps = 8;
-constexpr int kThreads = 32 * (2 + kConvWarps);
-constexpr int kStageV = 32;                  // vertices per pipeline stage (one 128-byte row of FP32)
-constexpr uint32_t kBoxBytes = 32 * 128;     // one TMA box: 32 vertices x 32 FP32 (features or basis)
-constexpr uint32_t kGroupBytes = 4 * kBoxBytes;   // 128 features of one stage
+constexpr int kFWarps = 8, kPWarps = 4;
+constexpr int kThreads = 32 * (2 + kFWarps + kPWarps);
+constexpr int kStageV = 32;                       // vertices per pipeline stage
+constexpr int kStepV = 16;                        // vertices per K-step (one slot)
+constexpr uint32_t kBoxBytes = kStageV * 128;     // one TMA box: 32 vertices x 32 FP32 (features or basis)
+constexpr uint32_t kColBytes = kStepV * 128;      // 16 vertices x 64 basis functions of one third
 
-constexpr int kMaxFg = 2;   // feature groups of 128 per CTA (the planner caps FP32 units at 2)
+// (a, b) -> heads, middles and tails, each pair packed low = a, high = b.
+__device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  a -= __uint_as_float(hi << 16); b -= __uint_as_float(hi & 0xffff0000u);
+  const __nv_bfloat162 m = __floats2bfloat162_rn(a, b);
+  mid = *reinterpret_cast<const uint32_t*>(&m);
+  a -= __uint_as_float(mid << 16); b -= __uint_as_float(mid & 0xffff0000u);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(a, b);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// The whole warp waits and goes on, or gives up, together.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort));
+}
+
+// The MMAs of one segment of kFg feature groups and kAccs accumulators each. One thread issues them,
+// and at small k the time it takes per MMA counts: everything but the waits is computed beforehand.
+template <int kFg, int kAccs>
+__device__ __forceinline__ bool issue(const TcProjParams& P, const TcItem& item, int nst, uint32_t tmem_base, uint8_t* sB,
+                                      uint64_t* part_full, uint64_t* part_empty, uint32_t& phase, volatile int* abort) {
+  const bool lead = (threadIdx.x & 31) == 0;
+  const uint32_t npad = (uint32_t)item.npad;
+  const uint32_t i1 = tc::idesc_bf16_f32(128, npad, 0, 1);
+  const uint32_t i2 = tc::idesc_bf16_f32(128, 2 * npad, 0, 1), i3 = tc::idesc_bf16_f32(128, 3 * npad, 0, 1);
+  const uint64_t third = (uint64_t)(((npad + 63) / 64) * kColBytes) >> 4;      // in descriptor units
+  uint64_t bh[kTc32Slots];
+#pragma unroll
+  for (int q = 0; q < kTc32Slots; ++q)
+    bh[q] = tc::smem_desc(tc::smem_u32(sB + (size_t)q * P.part_bytes), kColBytes, 1024, tc::kLayoutSW128);
+  for (int st = 0; st < nst; ++st) {
+#pragma unroll
+    for (int q = 0; q < kTc32Slots; ++q) {
+      if (!warp_wait(&part_full[q], phase, abort)) return false;
+      tc::tc_fence_after();
+      const uint32_t on = st == 0 && q == 0 ? 0u : 1u;
+#pragma unroll
+      for (int m = 0; m < kFg; ++m) {
+        const uint32_t a = tmem_base + (uint32_t)(512 - (q * kFg + m + 1) * kTc32SlotCols);
+        const uint32_t d = tmem_base + (uint32_t)(m * kAccs) * npad;
+        if (kAccs == 3) {                 // [Ph | Pm | Pl] side by side
+          if (lead) tc::mma_bf16_ta(d, a, bh[q], i3, on);
+          if (lead) tc::mma_bf16_ta(d + npad, a + 8, bh[q], i2, 1u);
+          if (lead) tc::mma_bf16_ta(d + 2 * npad, a + 16, bh[q], i1, 1u);
+        } else {
+          const uint32_t e = d + (uint32_t)(kAccs - 1) * npad;
+          if (lead) tc::mma_bf16_ta(d, a, bh[q], i1, on);
+          if (lead) tc::mma_bf16_ta(e, a, bh[q] + third, i1, kAccs == 2 ? on : 1u);
+          if (lead) tc::mma_bf16_ta(e, a, bh[q] + 2 * third, i1, 1u);
+          if (lead) tc::mma_bf16_ta(e, a + 8, bh[q], i1, 1u);
+          if (lead) tc::mma_bf16_ta(e, a + 8, bh[q] + third, i1, 1u);
+          if (lead) tc::mma_bf16_ta(e, a + 16, bh[q], i1, 1u);
+        }
+      }
+      if (lead) tc::mma_commit(&part_empty[q]);
+    }
+    phase ^= 1;
+  }
+  return true;
+}
 
 __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int S = P.stages;
-  // per stage: [F tile | Fl] (f_stage_bytes = 2 * fg * kGroupBytes), then [Phi | Ph | Pl]
   uint8_t* sF = smem;
   uint8_t* sP = sF + (size_t)S * P.f_stage_bytes;
-  float* sM = reinterpret_cast<float*>(sP + (size_t)S * P.p_stage_bytes);   // 32 masses per stage
+  uint8_t* sB = sP + (size_t)S * P.p_stage_bytes;                            // kTc32Slots slots
+  float* sM = reinterpret_cast<float*>(sB + (size_t)kTc32Slots * P.part_bytes);   // 32 masses per stage
   uint64_t* bars = reinterpret_cast<uint64_t*>(sM + (size_t)S * kStageV);
-  uint64_t* full_f = bars;
-  uint64_t* full_p = bars + S;
-  uint64_t* empty = bars + 2 * S;
-  uint64_t* acc_full = bars + 3 * S;    // [2]: accumulators double-buffered in TMEM
-  uint64_t* acc_empty = acc_full + 2;   // [2]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  uint64_t* full = bars;                // [S] F, Phi and masses have landed
+  uint64_t* empty = bars + S;           // [S] every converter has read them
+  uint64_t* part_full = bars + 2 * S;   // [kTc32Slots] the thirds are in place
+  uint64_t* part_empty = part_full + kTc32Slots;   // the MMAs have read them
+  uint64_t* acc_full = part_empty + kTc32Slots;
+  uint64_t* acc_empty = acc_full + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      tc::mbar_init(&full_f[s], 1);
-      tc::mbar_init(&full_p[s], kConvWarps);
-      tc::mbar_init(&empty[s], 1);
+      tc::mbar_init(&full[s], 1);
+      tc::mbar_init(&empty[s], kFWarps + kPWarps);
     }
-    for (int b = 0; b < 2; ++b) {
-      tc::mbar_init(&acc_full[b], 1);
-      tc::mbar_init(&acc_empty[b], kConvWarps);
+    for (int q = 0; q < kTc32Slots; ++q) {
+      tc::mbar_init(&part_full[q], kFWarps + kPWarps);
+      tc::mbar_init(&part_empty[q], 1);
     }
+    tc::mbar_init(acc_full, 1);
+    tc::mbar_init(acc_empty, kFWarps);
     *abort_flag = 0;
     tc::fence_mbar_init();
   }
@@ -79,36 +154,41 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    // each lane issues its own boxes: one lane issuing all of a stage's takes longer than the copies
+    {
       uint32_t stage = 0, phase = 0;
       for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
         const TcItem item = P.items[it];
         const CUtensorMap* fmap = P.fmaps + item.shape;
         const CUtensorMap* pmap = P.phimaps + item.shape;
         const CUtensorMap* mmap = P.massmaps + item.shape;
-        tc::prefetch_tmap(fmap);
-        tc::prefetch_tmap(pmap);
-        tc::prefetch_tmap(mmap);
         const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
-        const int kb = (item.npad + 31) / 32;
-        const uint32_t bytes = (uint32_t)item.fg * kGroupBytes + (uint32_t)kb * kBoxBytes + kStageV * 4;
+        const int nf = item.fg * 4, kb = (item.npad + 31) / 32;
+        const uint32_t bytes = (uint32_t)(nf + kb) * kBoxBytes + kStageV * 4;
+        if (lane == 0) {
+          tc::prefetch_tmap(fmap);
+          tc::prefetch_tmap(pmap);
+          tc::prefetch_tmap(mmap);
+        }
         for (int st = 0; st < nst; ++st) {
-          if (!tc::mbar_wait(&empty[stage], phase ^ 1, abort_flag)) goto producer_done;
-          tc::mbar_arrive_expect_tx(&full_f[stage], bytes);
-          uint8_t* dst = sF + (size_t)stage * P.f_stage_bytes;
-          uint8_t* pdst = sP + (size_t)stage * P.p_stage_bytes;
+          if (!warp_wait(&empty[stage], phase ^ 1, abort_flag)) goto producer_done;
+          if (lane == 0) tc::mbar_arrive_expect_tx(&full[stage], bytes);
+          __syncwarp();
           const int y = (int)(item.v0 + (int64_t)st * kStageV);
-          for (int m = 0; m < item.fg; ++m)
-            for (int h = 0; h < 4; ++h)
-              tc::tma_load_2d(dst + (m * 4 + h) * kBoxBytes, fmap, &full_f[stage], item.f0 + m * 128 + h * 32, y);
-          for (int b = 0; b < kb; ++b)
-            tc::tma_load_2d(pdst + b * kBoxBytes, pmap, &full_f[stage], item.n0 + b * 32, y);
-          tc::tma_load_1d(sM + (size_t)stage * kStageV, mmap, &full_f[stage], y);
+          if (lane < nf) {
+            tc::tma_load_2d(sF + (size_t)stage * P.f_stage_bytes + lane * kBoxBytes, fmap, &full[stage],
+                            item.f0 + lane * 32, y);
+          } else if (lane < nf + kb) {
+            const int b = lane - nf;
+            tc::tma_load_2d(sP + (size_t)stage * P.p_stage_bytes + b * kBoxBytes, pmap, &full[stage], item.n0 + b * 32, y);
+          } else if (lane == 31) {
+            tc::tma_load_1d(sM + (size_t)stage * kStageV, mmap, &full[stage], y);
+          }
           if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
         }
       }
     producer_done:
-      if (*abort_flag) {
+      if (lane == 0 && *abort_flag) {
         // let copies already in flight land before the CTA's shared memory goes away
         const uint64_t t0 = tc::globaltimer();
         while (tc::globaltimer() - t0 < 2000000ull) {}
@@ -116,147 +196,106 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0;
-      uint32_t acc_phase[2] = {0, 0};
-      int buf = 0;
-      const uint32_t half_cols = P.tmem_cols / 2;
+    {
+      uint32_t phase = 0, acc_phase = 0;
       for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
         const TcItem item = P.items[it];
-        if (!tc::mbar_wait(&acc_empty[buf], acc_phase[buf] ^ 1, abort_flag)) break;
+        if (!warp_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
         tc::tc_fence_after();
-        const uint32_t idesc = tc::idesc_tf32(128, (uint32_t)item.npad);
         const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
-        const int kb = (item.npad + 31) / 32;
-        bool ok = true;
-        for (int st = 0; st < nst && ok; ++st) {
-          ok = tc::mbar_wait(&full_f[stage], phase, abort_flag) && tc::mbar_wait(&full_p[stage], phase, abort_flag);
-          if (!ok) break;
-          tc::tc_fence_after();
-          const uint32_t f_base = tc::smem_u32(sF + (size_t)stage * P.f_stage_bytes);
-          const uint32_t fl_base = f_base + (uint32_t)item.fg * kGroupBytes;
-          const uint32_t ph = tc::smem_u32(sP + (size_t)stage * P.p_stage_bytes) + (uint32_t)kb * kBoxBytes;
-          const uint32_t pl = ph + (uint32_t)item.npad * 128u;
-#pragma unroll
-          for (int kk = 0; kk < kStageV / 8; ++kk) {
-            const uint64_t bh = tc::smem_desc(ph + kk * 32, 16, 1024, tc::kLayoutSW128);
-            const uint64_t bl = tc::smem_desc(pl + kk * 32, 16, 1024, tc::kLayoutSW128);
-            for (int m = 0; m < item.fg; ++m) {
-              const uint64_t af = tc::smem_desc(f_base + m * kGroupBytes + kk * 32, 16, 1024, tc::kLayoutSW128);
-              const uint64_t al = tc::smem_desc(fl_base + m * kGroupBytes + kk * 32, 16, 1024, tc::kLayoutSW128);
-              const uint32_t d = tmem_base + (uint32_t)buf * half_cols + (uint32_t)(m * item.npad);
-              tc::mma_tf32(d, af, bh, idesc, (st | kk) != 0 ? 1u : 0u);
-              tc::mma_tf32(d, af, bl, idesc, 1u);
-              tc::mma_tf32(d, al, bh, idesc, 1u);
-            }
-          }
-          tc::mma_commit(&empty[stage]);
-          if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
+        const int accs = tc32_accs(item.fg, item.npad);
+        bool ok;
+        if (accs == 3) {
+          ok = item.fg == 2 ? issue<2, 3>(P, item, nst, tmem_base, sB, part_full, part_empty, phase, abort_flag)
+                            : issue<1, 3>(P, item, nst, tmem_base, sB, part_full, part_empty, phase, abort_flag);
+        } else if (accs == 2) {
+          ok = item.fg == 2 ? issue<2, 2>(P, item, nst, tmem_base, sB, part_full, part_empty, phase, abort_flag)
+                            : issue<1, 2>(P, item, nst, tmem_base, sB, part_full, part_empty, phase, abort_flag);
+        } else {
+          ok = item.fg == 2 ? issue<2, 1>(P, item, nst, tmem_base, sB, part_full, part_empty, phase, abort_flag)
+                            : issue<1, 1>(P, item, nst, tmem_base, sB, part_full, part_empty, phase, abort_flag);
         }
         if (!ok) break;
-        tc::mma_commit(&acc_full[buf]);
-        acc_phase[buf] ^= 1;
-        buf ^= 1;
+        if (lane == 0) tc::mma_commit(acc_full);
+        acc_phase ^= 1;
       }
     }
-  } else {
-    // ------------------------------------------------------------ converters + epilogue
-    const int ct = threadIdx.x - 64;   // 0 .. 255
-    const int cw = warp - 2;
-    uint32_t stage = 0, phase = 0;
-    uint32_t acc_phase[2] = {0, 0};
-    int buf = 0;
-    const uint32_t half_cols = P.tmem_cols / 2;
+  } else if (warp < 2 + kFWarps) {
+    // ------------------------------------------------------------ thirds of F, epilogue
+    const int quarter = warp & 3, set = (warp - 2) >> 2;
+    const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    uint32_t off[8];                      // this lane's feature in vertex row i of an 8-row swizzle atom
+#pragma unroll
+    for (int i = 0; i < 8; ++i) off[i] = (uint32_t)i * 128u + ((uint32_t)((lane >> 2) ^ i) << 4) + (uint32_t)(lane & 3) * 4u;
+    uint32_t stage = 0, phase = 0, slot = 0, slot_phase = 0, acc_phase = 0;
     for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
       const TcItem item = P.items[it];
       const ShapeDev s = P.shapes[item.shape];
       const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
-      const int kb = (item.npad + 31) / 32;
+      // two feature groups: one each for the two sets of four warps; one group: 8 vertices each
+      const bool two = item.fg == 2;
+      const int m = two ? set : 0;
+      const uint32_t c0 = two ? 0u : (uint32_t)set;
       for (int st = 0; st < nst; ++st) {
-        if (!tc::mbar_wait(&full_f[stage], phase, abort_flag)) goto conv_done;
-        uint8_t* ftile = sF + (size_t)stage * P.f_stage_bytes;
-        uint8_t* phi = sP + (size_t)stage * P.p_stage_bytes;
-        uint8_t* th = phi + (size_t)kb * kBoxBytes;
-        uint8_t* tl = th + (size_t)item.npad * 128;
-        const float* mst = sM + (size_t)stage * kStageV;
-        const int64_t vbase = item.v0 + (int64_t)st * kStageV;
-        // F: read this thread's chunks (feature row f, vertices 4c .. 4c+3) out of the
-        // vertex-row TMA boxes, then (after every converter has read) write Fh in place and
-        // Fl beside it as K-major 128-byte-swizzled A tiles (row f, 32 vertices). The 32
-        // lanes of a warp take 32 consecutive features of one box and one vertex quad, so
-        // each read touches 32 distinct banks.
-        float fx[kMaxFg * 4][4];
-        const int nfc = item.fg * 128 * 8;
+        if (!warp_wait(&full[stage], phase, abort_flag)) goto done;
+        const uint8_t* tile = sF + (size_t)stage * P.f_stage_bytes + (m * 4 + quarter) * kBoxBytes + c0 * 1024;
 #pragma unroll
-        for (int r = 0; r < kMaxFg * 4; ++r) {
-          const int q = ct + 32 * kConvWarps * r;
-          if (q < nfc) {
-            const int c = (q >> 5) & 7, box = q >> 8;
-            const int ff = q & 31, f = 32 * box + ff;
+        for (int step = 0; step < kStageV / kStepV; ++step) {
+          float x[16];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int v = 4 * c + j;
-              fx[r][j] = *reinterpret_cast<const float*>(ftile + box * kBoxBytes + v * 128 +
-                                                         ((((ff >> 2) ^ (v & 7)) << 4) | ((ff & 3) << 2)));
-            }
+          for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const float*>(tile + step * 2048 + off[i]);
+          if (two) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[8 + i] = *reinterpret_cast<const float*>(tile + step * 2048 + 1024 + off[i]);
           }
-        }
-        tc::named_barrier_sync(1, 32 * kConvWarps);
+          uint32_t h[4], md[4], l[4];
 #pragma unroll
-        for (int r = 0; r < kMaxFg * 4; ++r) {
-          const int q = ct + 32 * kConvWarps * r;
-          if (q < nfc) {
-            const int c = (q >> 5) & 7, f = 32 * (q >> 8) + (q & 31);
-            float h[4], l[4];
+          for (int i = 0; i < 4; ++i) split3(x[2 * i], x[2 * i + 1], h[i], md[i], l[i]);
+          if (!warp_wait(&part_empty[slot], slot_phase ^ 1, abort_flag)) goto done;
+          tc::tc_fence_after();
+          const uint32_t a = lane_base + 512u - (uint32_t)((slot * item.fg + m + 1) * kTc32SlotCols) + c0 * 4;
+          tc::tmem_st4(a, h);
+          tc::tmem_st4(a + 8, md);
+          tc::tmem_st4(a + 16, l);
+          if (two) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              h[j] = tc::tf32_rna(fx[r][j]);
-              l[j] = fx[r][j] - h[j];
-            }
-            const uint32_t off = (uint32_t)f * 128u + ((uint32_t)(c ^ (f & 7)) << 4);
-            *reinterpret_cast<float4*>(ftile + off) = make_float4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<float4*>(ftile + (size_t)item.fg * kGroupBytes + off) = make_float4(l[0], l[1], l[2], l[3]);
+            for (int i = 0; i < 4; ++i) split3(x[8 + 2 * i], x[9 + 2 * i], h[i], md[i], l[i]);
+            tc::tmem_st4(a + 4, h);
+            tc::tmem_st4(a + 12, md);
+            tc::tmem_st4(a + 20, l);
           }
-        }
-        // Ph, Pl: 16-byte chunk (row n, vertices 4c .. 4c+3) of the K-major swizzled B tiles;
-        // a warp takes 32 consecutive basis functions of one box and one vertex quad
-        for (int q = ct; q < kb * 32 * 8; q += 32 * kConvWarps) {
-          const int n = 32 * (q >> 8) + (q & 31), c = (q >> 5) & 7;
-          if (n >= item.npad) continue;
-          float hv[4], lv[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int v = 4 * c + j;
-            const int b = n >> 5, nn = n & 31;
-            const float ph = *reinterpret_cast<const float*>(phi + b * kBoxBytes + v * 128 +
-                                                             ((((nn >> 2) ^ (v & 7)) << 4) | ((nn & 3) << 2)));
-            const float p = (vbase + v < item.v1) ? ph * mst[v] : 0.f;
-            hv[j] = tc::tf32_rna(p);
-            lv[j] = p - hv[j];
+          if (step == kStageV / kStepV - 1) {
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&empty[stage]);
           }
-          const uint32_t off = (uint32_t)n * 128u + ((uint32_t)(c ^ (n & 7)) << 4);
-          *reinterpret_cast<float4*>(th + off) = make_float4(hv[0], hv[1], hv[2], hv[3]);
-          *reinterpret_cast<float4*>(tl + off) = make_float4(lv[0], lv[1], lv[2], lv[3]);
+          tc::tmem_st_wait();
+          tc::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&part_full[slot]);
+          if (++slot == (uint32_t)kTc32Slots) { slot = 0; slot_phase ^= 1; }
         }
-        tc::fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&full_p[stage]);
         if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
       }
-      // epilogue: accumulators -> this item's partial A (nk x stride, row-major)
-      if (!tc::mbar_wait(&acc_full[buf], acc_phase[buf], abort_flag)) goto conv_done;
+      // accumulators -> this item's partial A (nk x stride, row-major)
+      if (!warp_wait(acc_full, acc_phase, abort_flag)) goto done;
       tc::tc_fence_after();
       {
-        const int quarter = warp & 3, half = cw >> 2;
+        const int accs = tc32_accs(item.fg, item.npad);
         const int stride = item.fg * 128;
         float* part = P.ws + item.part_off;
-        for (int m = 0; m < item.fg; ++m) {
-          const int fl = m * 128 + quarter * 32 + lane;
+        for (int g = 0; g < item.fg; ++g) {
+          const int fl = g * 128 + quarter * 32 + lane;
           const bool fok = item.f0 + fl < s.d;
-          for (int ch = half; ch < item.npad / 16; ch += 2) {
+          for (int ch = set; ch < item.npad / 16; ch += 2) {
+            const uint32_t d = lane_base + (uint32_t)(g * accs * item.npad + ch * 16);
             float v[16];
-            tc::tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * half_cols +
-                              (uint32_t)(m * item.npad + ch * 16), v);
+            tc::tmem_ld16(d, v);
+            for (int r = 1; r < accs; ++r) {
+              float w[16];
+              tc::tmem_ld16(d + r * item.npad, w);
+#pragma unroll
+              for (int t = 0; t < 16; ++t) v[t] += w[t];
+            }
             if (fok) {
 #pragma unroll
               for (int t = 0; t < 16; ++t) {
@@ -269,12 +308,82 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
       }
       tc::tc_fence_before();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&acc_empty[buf]);
-      acc_phase[buf] ^= 1;
-      buf ^= 1;
+      if (lane == 0) tc::mbar_arrive(acc_empty);
+      acc_phase ^= 1;
     }
-  conv_done:;
+  } else {
+    // ------------------------------------------------------------ thirds of P
+    const int pt = threadIdx.x - 32 * (2 + kFWarps);   // 0 .. 127
+    // 8 lanes read 64 columns of one vertex row, 8 each: the two boxes' lanes take their two
+    // 16-byte chunks in opposite order, so that each read touches 32 distinct banks
+    const int j = pt & 7, v = pt >> 3, swap = j >> 2;
+    const uint32_t row = (uint32_t)swap * kBoxBytes + (uint32_t)v * 128u;
+    const uint32_t ca = row + ((uint32_t)((2 * (j & 3) + swap) ^ (v & 7)) << 4);
+    const uint32_t cb = row + ((uint32_t)((2 * (j & 3) + (swap ^ 1)) ^ (v & 7)) << 4);
+    uint32_t stage = 0, phase = 0, slot = 0, slot_phase = 0;
+    for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
+      const TcItem item = P.items[it];
+      const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
+      const int ng = (item.npad + 63) / 64;
+      // chunk of 8 columns p * stride + j of the slot: the thirds side by side, or 64-column aligned
+      const int stride = tc32_accs(item.fg, item.npad) == 3 ? item.npad / 8 : ng * 8;
+      uint32_t dst[3];
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        const int ci = p * stride + j;
+        dst[p] = (uint32_t)(ci >> 3) * kColBytes + (uint32_t)v * 128u + ((uint32_t)((ci ^ v) & 7) << 4);
+      }
+      for (int st = 0; st < nst; ++st) {
+        if (!warp_wait(&full[stage], phase, abort_flag)) goto done;
+#pragma unroll
+        for (int step = 0; step < kStageV / kStepV; ++step) {
+          const uint8_t* phi = sP + (size_t)stage * P.p_stage_bytes + step * kStepV * 128;
+          uint8_t* out = sB + (size_t)slot * P.part_bytes;
+          const int vs = step * kStepV + v;
+          const float mv = item.v0 + (int64_t)st * kStageV + vs < item.v1 ? sM[(size_t)stage * kStageV + vs] : 0.f;
+          // columns 64 g0 .. 64 g0 + 127: both groups' reads first
+          for (int g0 = 0; g0 < ng; g0 += 2) {
+            float4 x[2], y[2];
+            bool on[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              on[e] = (g0 + e) * 64 + j * 8 < item.npad;
+              x[e] = y[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (on[e]) {
+                x[e] = *reinterpret_cast<const float4*>(phi + (g0 + e) * 2 * kBoxBytes + ca);
+                y[e] = *reinterpret_cast<const float4*>(phi + (g0 + e) * 2 * kBoxBytes + cb);
+              }
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              if (g0 + e >= ng) break;
+              const float4 p = swap ? y[e] : x[e], q = swap ? x[e] : y[e];
+              uint4 h, md, l;
+              split3(p.x * mv, p.y * mv, h.x, md.x, l.x);
+              split3(p.z * mv, p.w * mv, h.y, md.y, l.y);
+              split3(q.x * mv, q.y * mv, h.z, md.z, l.z);
+              split3(q.z * mv, q.w * mv, h.w, md.w, l.w);
+              if (g0 + e == 0 && !warp_wait(&part_empty[slot], slot_phase ^ 1, abort_flag)) goto done;
+              if (on[e]) {
+                *reinterpret_cast<uint4*>(out + (g0 + e) * kColBytes + dst[0]) = h;
+                *reinterpret_cast<uint4*>(out + (g0 + e) * kColBytes + dst[1]) = md;
+                *reinterpret_cast<uint4*>(out + (g0 + e) * kColBytes + dst[2]) = l;
+              }
+            }
+          }
+          tc::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            if (step == kStageV / kStepV - 1) tc::mbar_arrive(&empty[stage]);
+            tc::mbar_arrive(&part_full[slot]);
+          }
+          if (++slot == (uint32_t)kTc32Slots) { slot = 0; slot_phase ^= 1; }
+        }
+        if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
+      }
+    }
   }
+done:
 
   __syncthreads();
   if (warp == 1) tc::tmem_dealloc(tmem_base, P.tmem_cols);
