@@ -27,10 +27,8 @@ int32_t cuda_fail(cudaError_t e, const char* where) {
 constexpr int64_t kAlignFloats = 64;   // 256-byte alignment of workspace regions
 constexpr int64_t kTcChunkV = 8192;    // vertices per work item of the tensor-core backward projection
 constexpr int kTcCtas = 152;           // persistent CTAs of the projection (one per GB300 SM)
-constexpr int64_t kStageV = 64;        // vertices per projection pipeline stage
 constexpr int64_t kTcSegMaxV = 8192;   // longest projection segment (one TMEM accumulation), BF16 F
 constexpr int64_t kTc32SegMaxV[3] = {512, 2048, 2048};   // the same for FP32 F, by its accumulators
-constexpr int64_t kTc32StageV = 32;    // vertices per stage, FP32 F
 constexpr int kSmemBudget = 227 * 1024;
 
 int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
@@ -67,7 +65,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 // One launch of the forward projection: the segments of one spectral-size class.
 struct TcLaunch {
   int32_t cta_off;     // offset of its proj_ctas + 1 CTA boundaries in tc_cta_first
-  int32_t stages;
+  int32_t stages, stage_v;
   uint32_t f_stage, p_stage, part, tmem_cols;
   int32_t smem;
 };
@@ -246,8 +244,6 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
     // FP32-feature kernel keeps the chain in the FP32 class: 2048 vertices (128 adds) where the
     // heads' products have an accumulator of their own, 512 (192 adds) where they share it.
     // The tuning knob applies to BF16 features.
-    // vertices per pipeline stage: 64 (BF16 F, one 128-byte row of BF16) or 32 (FP32 F)
-    const int64_t stage_v = P.tc32 ? kTc32StageV : kStageV;
     for (int cls = 0; cls < 4; ++cls) {
       const std::vector<Unit>& units = classes[cls];
       if (units.empty()) continue;
@@ -255,15 +251,20 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
       double total = 0.0;
       for (const Unit& u : units) {
         total += u.cpv * (double)P.shapes[u.s].n;
-        // BF16: F tile; Phi tile converted in place into P hi / lo.
-        // FP32: F and Phi tiles of 32 vertices; the basis parts have slots of their own.
+        // Bytes of a vertex. BF16: F tile; Phi tile converted in place into P hi / lo.
+        // FP32: F and Phi tiles; the basis parts have slots of their own.
         const uint32_t kbu = (uint32_t)((u.npad + 31) / 32);
-        fmax = std::max<uint32_t>(fmax, (uint32_t)u.fg * 16384u);
-        const uint32_t pb = P.tc32 ? kbu * 4096u : std::max<uint32_t>(kbu * 8192u, (uint32_t)u.npad * 256u);
-        pmax = std::max<uint32_t>(pmax, pb);
+        fmax = std::max<uint32_t>(fmax, (uint32_t)u.fg * (P.tc32 ? 512u : 256u));
+        pmax = std::max<uint32_t>(pmax, kbu * 128u);
         if (P.tc32) part = std::max<uint32_t>(part, 3u * (uint32_t)((u.npad + 63) / 64) * 2048u);
         tmax = std::max<uint32_t>(tmax, (uint32_t)(u.fg * u.npad) * (tc_merged(u.fg, u.npad) ? 2u : 1u));
       }
+      // Vertices per stage. BF16 F: 64, a 128-byte row of P hi and one of P lo; 32, hi and lo halves
+      // of a row, where three stages of 64 do not fit (8 shapes of n = 200000, k = 200, d = 512:
+      // two of 64 763 us, five of 32 670; 64 shapes of n = 50000, k = 300, d = 256, where three
+      // fit: 1240 against 1355)
+      const bool three = 3u * 64u * (fmax + pmax + 4u) + 1536u <= (uint32_t)kSmemBudget;
+      const int64_t stage_v = P.tc32 || !three ? 32 : 64;
       TcLaunch L{};
       L.cta_off = (int32_t)P.tc_cta_first.size();
       const int nctas = P.proj_ctas;
@@ -310,8 +311,9 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
         P.tc_max_group_elems = std::max<int64_t>(P.tc_max_group_elems, (int64_t)u.nk * rg.dspan);
       }
       for (int c = cta + 1; c <= nctas; ++c) first[c] = (int32_t)P.tc_items.size();
-      L.f_stage = P.tc32 ? fmax : std::max<uint32_t>(fmax, 16384u);
-      L.p_stage = P.tc32 ? pmax : (std::max<uint32_t>(pmax, 8192u) + 1023u) / 1024u * 1024u;
+      L.f_stage = fmax * (uint32_t)stage_v;
+      L.p_stage = pmax * (uint32_t)stage_v;
+      L.stage_v = (int32_t)stage_v;
       L.part = part;
       uint32_t cols = P.tc32 ? 512 : 32;   // FP32: accumulators and operand slots
       while (cols < tmax) cols <<= 1;
@@ -759,9 +761,9 @@ int32_t fmap_batch_create(fmap_ctx* ctx, const fmap_shape_desc* shapes, int32_t 
     if (!encode) { cudaFree(b->dev_mem); delete b; return cuda_fail(cudaErrorNotSupported, "cuTensorMapEncodeTiled"); }
     for (int s = 0; s < n_shapes; ++s) {
       const ShapeDev& sd = P.shapes[s];
-      // features: BF16 box 64 features x 64 vertices, or FP32 box 32 features x 32 vertices
-      // (a 128-byte row either way); the basis and mass boxes follow the stage length
-      const cuuint32_t sv = P.tc32 ? 32 : 64;
+      // features: box of 64 (BF16) or 32 (FP32) features, a 128-byte row either way, x 32 vertices,
+      // like the basis and mass boxes (a longer stage takes several)
+      const cuuint32_t sv = 32;
       CUtensorMap m;
       cuuint64_t gdim[2] = {(cuuint64_t)sd.d, (cuuint64_t)sd.n};
       cuuint64_t gstride[1] = {(cuuint64_t)sd.ld_feat * (P.tc32 ? 4 : 2)};
@@ -777,8 +779,7 @@ int32_t fmap_batch_create(fmap_ctx* ctx, const fmap_shape_desc* shapes, int32_t 
         return FMAP_ERR_CUDA;
       }
       put(o_tm + s * (int64_t)sizeof(CUtensorMap), &m, sizeof(m));
-      // FP32 basis, box 32 basis x sv vertices (the forward projection's tiles and, at 64
-      // vertices, the halves of the backward projection's 128-vertex tiles)
+      // FP32 basis, box 32 basis x sv vertices (the forward projection's tiles)
       CUtensorMap pm;
       cuuint64_t pdim[2] = {(cuuint64_t)sd.k, (cuuint64_t)sd.n};
       cuuint64_t pstride[1] = {(cuuint64_t)sd.ld_phi * 4};
@@ -958,6 +959,7 @@ int32_t fmap_project(fmap_batch* b, float* a_out, void* ws, size_t ws_bytes, voi
     tp.items = b->d_tc_items;
     tp.cta_first = b->d_tc_cta_first + L.cta_off;
     tp.stages = L.stages;
+    tp.stage_v = L.stage_v;
     tp.f_stage_bytes = L.f_stage;
     tp.p_stage_bytes = L.p_stage;
     tp.part_bytes = L.part;

@@ -122,13 +122,14 @@ __host__ __device__ __forceinline__ bool tc_merged(int fg, int npad) { return np
 
 struct TcProjParams {
   const ShapeDev* shapes;
-  const CUtensorMap* fmaps;     // per shape: features, BF16 box 64 x 64 or FP32 box 32 x 32 (features x
+  const CUtensorMap* fmaps;     // per shape: features, BF16 box 64 x 32 or FP32 box 32 x 32 (features x
                                 //   vertices), 128-byte swizzle
-  const CUtensorMap* phimaps;   // per shape: FP32 basis, box 32 basis x (64 or 32) vertices, 128-byte swizzle
-  const CUtensorMap* massmaps;  // per shape: FP32 mass, 1-D box of 64 or 32
+  const CUtensorMap* phimaps;   // per shape: FP32 basis, box 32 basis x 32 vertices, 128-byte swizzle
+  const CUtensorMap* massmaps;  // per shape: FP32 mass, 1-D box of 32
   const TcItem* items;          // segments, grouped by CTA
   const int32_t* cta_first;     // CTA c owns segments [cta_first[c], cta_first[c + 1])
   int32_t stages;
+  int32_t stage_v;            // BF16 features: vertices per stage, 64 or 32
   uint32_t f_stage_bytes;
   uint32_t p_stage_bytes;
   uint32_t part_bytes;        // FP32 features: one slot of the basis parts
@@ -186,7 +187,6 @@ cudaError_t launch_project_bwd_tc32(const TcBwdParams& p, int grid, int smem_byt
 cudaError_t project_tc_set_smem(int bytes);
 cudaError_t project_tc32_set_smem(int bytes);
 cudaError_t launch_project_tc32(const TcProjParams& p, int grid, int smem_bytes, cudaStream_t st);
-int project_tc_threads();
 cudaError_t launch_project_tc(const TcProjParams& p, int grid, int smem_bytes, cudaStream_t st);
 cudaError_t launch_project_tc_reduce(const ShapeDev* shapes, const int64_t* parts, const TcRedGroup* groups,
                                      int n_groups, int64_t max_elems, float* a_out, const float* ws,

@@ -5,19 +5,23 @@
 // One persistent CTA per SM walks its own contiguous range of the batch's
 // (shape, feature group) vertex sequence (stream-K split into equal-cost
 // ranges); a range is cut into segments at shape / group boundaries and every
-// segment writes one partial A. Per 64-vertex stage:
+// segment writes one partial A. Per stage of 64 or 32 vertices:
 //   warp 0      TMA-loads the F tile (MN-major, 128-byte swizzle), the Phi tile
-//               (FP32, 32-column boxes, 128-byte swizzle) and the 64 masses;
+//               (FP32, 32-column boxes, 128-byte swizzle) and the masses;
 //   warps 2-9   read Phi and M from shared memory, form P = M * Phi in FP32 and
 //               split it into BF16 hi + lo (P = hi + lo to ~2^-17), written in place
 //               over the Phi tile as K-major 128-byte-swizzled B tiles: the mass is
 //               fused into the operand load;
 //   warp 1      issues tcgen05.mma (M = 128 features, K = 16 vertices) into FP32 accumulators
 //               in TMEM: N = k rounded up to 16 for hi and for lo, or, where the columns
-//               allow it (tc_merged), one MMA on the rows of hi and lo together, whose two
-//               accumulators the epilogue adds. An MMA of small N is bound by its reads of the F
-//               tile, which two MMAs take twice: 64 shapes of n = 50000, d = 256 at k = 30 /
-//               50 / 100 took 433 / 454 / 500 us with two and 380 / 405 / 470 with one.
+//               allow it (tc_merged, stages of 64), one MMA on the rows of hi and lo together,
+//               whose two accumulators the epilogue adds.
+// What bounds it: the reads of F and Phi (6.1 to 6.6 TB/s for most sizes); at small k the MMAs
+// come next, each of which reads the F tile and takes its time to issue. 64 shapes of n = 50000,
+// d = 256 at k = 30 / 50 / 100 / 200: 433 / 454 / 500 / 789 us with separate MMAs for hi and lo,
+// descriptors built between them, one lane issuing all copies and two stages of 64 vertices at
+// k = 200; 380 / 405 / 470 / 771 with one MMA; 335 / 367 / 445 / 658 with descriptors ahead of
+// the waits, a lane per copy and stages of 32 where three of 64 do not fit.
 // At the end of a segment warps 2-9 read the accumulators back (tcgen05.ld) and
 // write the segment's partial A; a second kernel adds the partials of each shape
 // in a fixed order. F is exact in BF16, so A carries only the ~2^-17 error of
@@ -34,9 +38,7 @@ namespace {
 
 constexpr int kConvWarps = 8;
 constexpr int kThreads = 32 * (2 + kConvWarps);
-constexpr int kStageV = 64;            // vertices per pipeline stage (= one 128-byte K row of bf16)
-constexpr uint32_t kBoxBytes = 64 * 64 * 2;   // one TMA box: 64 vertices x 64 features bf16
-constexpr uint32_t kPhiBoxBytes = 64 * 128;    // one TMA box: 64 vertices x 32 basis functions fp32
+constexpr uint32_t kBoxBytes = 32 * 128;       // one TMA box: 32 vertices x 64 features bf16, or x 32 basis functions fp32
 
 // (a, b) -> BF16 heads RN(a), RN(b) and remainders RN(a - head), RN(b - head), each pair
 // packed low = a, high = b (one packed conversion per pair).
@@ -48,13 +50,55 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint3
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
+// The whole warp waits and goes on, or gives up, together.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort));
+}
+
+// The MMAs of one segment. kV: vertices per stage; kFg: feature groups (0: item.fg); kMerged: tc_merged. One
+// lane issues them and the time per MMA counts at small k, so the descriptors are computed ahead of the waits.
+template <int kV, int kFg, bool kMerged>
+__device__ __forceinline__ bool issue(const TcProjParams& P, const TcItem& item, int nst, uint32_t tmem_base, uint8_t* sF,
+                                      uint8_t* sP, uint64_t* full_f, uint64_t* full_p, uint64_t* empty, uint32_t& stage,
+                                      uint32_t& phase, volatile int* abort) {
+  const bool lead = (threadIdx.x & 31) == 0;
+  const int fg = kFg ? kFg : item.fg;
+  const uint32_t npad = (uint32_t)item.npad;
+  const uint32_t cols = npad * (kMerged ? 2u : 1u);      // accumulator columns per feature group
+  const uint32_t idesc = tc::idesc_bf16_f32(128, cols, 1, 0);
+  const uint32_t lo = kV == 64 ? npad * 8 : 4;           // from P hi to P lo, in 16-byte units
+  for (int st = 0; st < nst; ++st) {
+    const uint64_t ad = tc::smem_desc(tc::smem_u32(sF + (size_t)stage * P.f_stage_bytes), kV * 128, 1024, tc::kLayoutSW128);
+    const uint64_t bd = tc::smem_desc(tc::smem_u32(sP + (size_t)stage * P.p_stage_bytes), 16, 1024, tc::kLayoutSW128);
+    if (!warp_wait(&full_f[stage], phase, abort) || !warp_wait(&full_p[stage], phase, abort)) return false;
+    tc::tc_fence_after();
+#pragma unroll
+    for (int kk = 0; kk < kV / 16; ++kk) {
+#pragma unroll
+      for (int m = 0; m < (kFg ? kFg : 4); ++m) {
+        if (m >= fg) break;
+        const uint64_t a = ad + ((m * 2 * kV * 128 + kk * 2048) >> 4), b = bd + ((kk * 32) >> 4);
+        const uint32_t d = tmem_base + (uint32_t)m * cols;
+        if (lead) {
+          tc::mma_bf16(d, a, b, idesc, (st | kk) != 0 ? 1u : 0u);
+          if (!kMerged) tc::mma_bf16(d, a, b + lo, idesc, 1u);
+        }
+      }
+    }
+    if (lead) tc::mma_commit(&empty[stage]);
+    if (++stage == (uint32_t)P.stages) { stage = 0; phase ^= 1; }
+  }
+  return true;
+}
+
+template <int kStageV>
 __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int S = P.stages;
   uint8_t* sF = smem;
   uint8_t* sP = sF + (size_t)S * P.f_stage_bytes;       // Phi tile, converted in place into P hi / lo
-  float* sM = reinterpret_cast<float*>(sP + (size_t)S * P.p_stage_bytes);   // 64 masses per stage
+  float* sM = reinterpret_cast<float*>(sP + (size_t)S * P.p_stage_bytes);   // kStageV masses per stage
   uint64_t* bars = reinterpret_cast<uint64_t*>(sM + (size_t)S * kStageV);
   uint64_t* full_f = bars;
   uint64_t* full_p = bars + S;
@@ -87,36 +131,45 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    // each lane issues its own boxes
+    {
       uint32_t stage = 0, phase = 0;
       for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
         const TcItem item = P.items[it];
         const CUtensorMap* fmap = P.fmaps + item.shape;
         const CUtensorMap* pmap = P.phimaps + item.shape;
         const CUtensorMap* mmap = P.massmaps + item.shape;
-        tc::prefetch_tmap(fmap);
-        tc::prefetch_tmap(pmap);
-        tc::prefetch_tmap(mmap);
         const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
-        const int kb = (item.npad + 31) / 32;
-        const uint32_t bytes = (uint32_t)item.fg * 2 * kBoxBytes + (uint32_t)kb * kPhiBoxBytes + kStageV * 4;
+        const int nf = item.fg * 2, kb = (item.npad + 31) / 32;     // at most 8 + 8 boxes
+        const uint32_t bytes = (uint32_t)(nf + kb) * (kStageV * 128) + kStageV * 4;
+        if (lane == 0) {
+          tc::prefetch_tmap(fmap);
+          tc::prefetch_tmap(pmap);
+          tc::prefetch_tmap(mmap);
+        }
         for (int st = 0; st < nst; ++st) {
-          if (!tc::mbar_wait(&empty[stage], phase ^ 1, abort_flag)) goto producer_done;
-          tc::mbar_arrive_expect_tx(&full_f[stage], bytes);
-          uint8_t* dst = sF + (size_t)stage * P.f_stage_bytes;
-          uint8_t* pdst = sP + (size_t)stage * P.p_stage_bytes;
+          if (!warp_wait(&empty[stage], phase ^ 1, abort_flag)) goto producer_done;
+          if (lane == 0) tc::mbar_arrive_expect_tx(&full_f[stage], bytes);
+          __syncwarp();
           const int y = (int)(item.v0 + (int64_t)st * kStageV);
-          for (int m = 0; m < item.fg; ++m)
-            for (int h = 0; h < 2; ++h)
-              tc::tma_load_2d(dst + (m * 2 + h) * kBoxBytes, fmap, &full_f[stage], item.f0 + m * 128 + h * 64, y);
-          for (int b = 0; b < kb; ++b)
-            tc::tma_load_2d(pdst + b * kPhiBoxBytes, pmap, &full_f[stage], item.n0 + b * 32, y);
-          tc::tma_load_1d(sM + (size_t)stage * kStageV, mmap, &full_f[stage], y);
+#pragma unroll
+          for (int h = 0; h < kStageV / 32; ++h) {
+            if (lane < nf) {
+              tc::tma_load_2d(sF + (size_t)stage * P.f_stage_bytes + lane * (kStageV * 128) + h * kBoxBytes, fmap,
+                              &full_f[stage], item.f0 + lane * 64, y + 32 * h);
+            } else if (lane < nf + kb) {
+              const int b = lane - nf;
+              tc::tma_load_2d(sP + (size_t)stage * P.p_stage_bytes + b * (kStageV * 128) + h * kBoxBytes, pmap,
+                              &full_f[stage], item.n0 + b * 32, y + 32 * h);
+            } else if (lane == 31) {
+              tc::tma_load_1d(sM + (size_t)stage * kStageV + 32 * h, mmap, &full_f[stage], y + 32 * h);
+            }
+          }
           if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
         }
       }
     producer_done:
-      if (*abort_flag) {
+      if (lane == 0 && *abort_flag) {
         // let copies already in flight land before the CTA's shared memory goes away
         const uint64_t t0 = tc::globaltimer();
         while (tc::globaltimer() - t0 < 2000000ull) {}
@@ -124,43 +177,26 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, acc_phase = 0;
-      for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
-        const TcItem item = P.items[it];
-        if (!tc::mbar_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
-        tc::tc_fence_after();
-        const bool merged = tc_merged(item.fg, item.npad);
-        const uint32_t cols = (uint32_t)item.npad * (merged ? 2u : 1u);      // accumulator columns per feature group
-        const uint32_t idesc = tc::idesc_bf16_f32(128, cols, 1, 0);
-        const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
-        bool ok = true;
-        for (int st = 0; st < nst && ok; ++st) {
-          ok = tc::mbar_wait(&full_f[stage], phase, abort_flag) && tc::mbar_wait(&full_p[stage], phase, abort_flag);
-          if (!ok) break;
-          tc::tc_fence_after();
-          const uint32_t a_base = tc::smem_u32(sF + (size_t)stage * P.f_stage_bytes);
-          const uint32_t ph = tc::smem_u32(sP + (size_t)stage * P.p_stage_bytes);
-          const uint32_t pl = ph + (uint32_t)item.npad * 128u;
-#pragma unroll
-          for (int kk = 0; kk < kStageV / 16; ++kk) {
-            const uint64_t bh = tc::smem_desc(ph + kk * 32, 16, 1024, tc::kLayoutSW128);
-            const uint64_t bl = tc::smem_desc(pl + kk * 32, 16, 1024, tc::kLayoutSW128);
-            for (int m = 0; m < item.fg; ++m) {
-              const uint64_t ad = tc::smem_desc(a_base + m * 2 * kBoxBytes + kk * 2048, kBoxBytes, 1024,
-                                                tc::kLayoutSW128);
-              const uint32_t d = tmem_base + (uint32_t)m * cols;
-              tc::mma_bf16(d, ad, bh, idesc, (st | kk) != 0 ? 1u : 0u);
-              if (!merged) tc::mma_bf16(d, ad, bl, idesc, 1u);
-            }
-          }
-          tc::mma_commit(&empty[stage]);
-          if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
-        }
-        if (!ok) break;
-        tc::mma_commit(acc_full);
-        acc_phase ^= 1;
+    uint32_t stage = 0, phase = 0, acc_phase = 0;
+    for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
+      const TcItem item = P.items[it];
+      if (!warp_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
+      tc::tc_fence_after();
+      const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
+      bool ok;
+      if constexpr (kStageV == 32) {
+        ok = item.fg == 2 ? issue<32, 2, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
+                          : issue<32, 0, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
+      } else if (tc_merged(item.fg, item.npad)) {
+        ok = item.fg == 1   ? issue<64, 1, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
+             : item.fg == 2 ? issue<64, 2, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
+                            : issue<64, 0, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
+      } else {
+        ok = issue<64, 0, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
       }
+      if (!ok) break;
+      if (lane == 0) tc::mma_commit(acc_full);
+      acc_phase ^= 1;
     }
   } else {
     // ------------------------------------------------------------ converters + epilogue
@@ -179,28 +215,29 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
         const float* mst = sM + (size_t)stage * kStageV;
         const int64_t vbase = item.v0 + (int64_t)st * kStageV;
         // read phase: unit (box b, row group c = 4 cg + csub, quad qs) = rows 8c..8c+7 x basis 32b+4qs..+3
-        float4 x[2][8];
+        float4 x[kStageV / 32][8];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
+        for (int r = 0; r < kStageV / 32; ++r) {
           const int wu = cw + kConvWarps * r;
-          if (wu < 2 * kb) {
-            const int b = wu >> 1, c = 4 * (wu & 1) + csub;
+          if (wu < kStageV / 32 * kb) {
+            const int b = kStageV == 64 ? wu >> 1 : wu, c = kStageV == 64 ? 4 * (wu & 1) + csub : csub;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               const int vl = 8 * c + i;
-              x[r][i] = *reinterpret_cast<const float4*>(tile + b * kPhiBoxBytes + vl * 128 + ((qs ^ (vl & 7)) << 4));
+              x[r][i] = *reinterpret_cast<const float4*>(tile + b * (kStageV * 128) + vl * 128 + ((qs ^ (vl & 7)) << 4));
             }
           }
         }
         tc::named_barrier_sync(1, 32 * kConvWarps);
-        // write phase: P hi at [0, npad*128), lo at [npad*128, 2*npad*128), K-major, 128-byte swizzle
+        // write phase, K-major, 128-byte swizzle: 64 vertices: P hi at [0, npad*128), lo at [npad*128, 2*npad*128);
+        // 32: hi in the first half of each row, lo in the second
         uint8_t* th = tile;
-        uint8_t* tl = tile + (size_t)item.npad * 128;
+        uint8_t* tl = kStageV == 64 ? tile + (size_t)item.npad * 128 : tile;
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
+        for (int r = 0; r < kStageV / 32; ++r) {
           const int wu = cw + kConvWarps * r;
-          if (wu < 2 * kb) {
-            const int b = wu >> 1, c = 4 * (wu & 1) + csub;
+          if (wu < kStageV / 32 * kb) {
+            const int b = kStageV == 64 ? wu >> 1 : wu, c = kStageV == 64 ? 4 * (wu & 1) + csub : csub;
             float mv[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) mv[i] = (vbase + 8 * c + i < item.v1) ? mst[8 * c + i] : 0.f;
@@ -223,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
               split_pair(pv[6], pv[7], hv.w, lv.w);
               const uint32_t off = (uint32_t)n * 128u + ((uint32_t)(c ^ (n & 7)) << 4);
               *reinterpret_cast<uint4*>(th + off) = hv;
-              *reinterpret_cast<uint4*>(tl + off) = lv;
+              *reinterpret_cast<uint4*>(tl + (kStageV == 64 ? off : off ^ 64u)) = lv;
             }
           }
         }
@@ -240,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
         const int quarter = warp & 3, half = cw >> 2;
         const int stride = item.fg * 128;
         float* part = P.ws + item.part_off;
-        const bool merged = tc_merged(item.fg, item.npad);
+        const bool merged = kStageV == 64 && tc_merged(item.fg, item.npad);
         const int cols = item.npad * (merged ? 2 : 1);
         for (int m = 0; m < item.fg; ++m) {
           const int fl = m * 128 + quarter * 32 + lane;
@@ -329,14 +366,15 @@ __global__ void __launch_bounds__(256) project_tc_reduce_kernel(const ShapeDev* 
 }  // namespace
 
 cudaError_t project_tc_set_smem(int bytes) {
-  return cudaFuncSetAttribute(project_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  const cudaError_t e = cudaFuncSetAttribute(project_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(project_tc_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
-
-int project_tc_threads() { return kThreads; }
 
 cudaError_t launch_project_tc(const TcProjParams& p, int grid, int smem_bytes, cudaStream_t st) {
   if (grid <= 0) return cudaSuccess;
-  project_tc_kernel<<<grid, kThreads, smem_bytes, st>>>(p);
+  if (p.stage_v == 64) project_tc_kernel<64><<<grid, kThreads, smem_bytes, st>>>(p);
+  else project_tc_kernel<32><<<grid, kThreads, smem_bytes, st>>>(p);
   return cudaGetLastError();
 }
 
