@@ -200,7 +200,7 @@ def algorithmic_work(wl, ir_steps, saved_k_max):
     bwd_bytes = sum(s.n * (4 * s.k + 4 + fsz * s.d) + 4 * s.k * s.d for s in wl.shapes)
     solve_flops, adj_flops, loss_flops, gemm_flops = 0.0, 0.0, 0.0, 0.0
     solve_bytes, adj_bytes = 0, 0
-    da_tiles = 0
+    gemm_blocks = 0
     for p in wl.pairs:
         # C is ky x k: ky row systems of size k (square maps: ky == k)
         k, ky = wl.shapes[p.x].k, wl.shapes[p.y].k
@@ -213,13 +213,13 @@ def algorithmic_work(wl, ir_steps, saved_k_max):
         # adjoint GEMMs: W = Gamma^T C + C^T Gamma, dA_y = Gamma A_x, dA_x = Gamma^T A_y - W A_x
         d = wl.shapes[p.x].d
         gemm_flops += 4.0 * k * k * ky + 2.0 * ky * k * d + 2.0 * k * (ky + k) * d
-        da_tiles += -(-k // 128) * -(-d // 128)
+        gemm_blocks = max(gemm_blocks, -(-max(2 * ky, k) // 32) + -(-(k + ky) // 32))
         # G, R and C move once each, saved factors written (forward) / read (adjoint)
         solve_bytes += 4 * (k * k + 2 * ky * k) + fac
         adj_bytes += 4 * 2 * ky * k + fac
     return dict(project=dict(bytes=proj_bytes, flops=proj_flops), project_bwd=dict(bytes=bwd_bytes, flops=proj_flops),
                 solve=dict(flops=solve_flops, bytes=solve_bytes), adj_solve=dict(flops=adj_flops, bytes=adj_bytes),
-                loss=dict(flops=loss_flops), adj_gemm=dict(flops=gemm_flops, da_tiles=da_tiles))
+                loss=dict(flops=loss_flops), adj_gemm=dict(flops=gemm_flops, blocks=gemm_blocks))
 
 
 # ---------------------------------------------------------------- oracle timing
@@ -622,18 +622,18 @@ def bench_workload(wid, args, dev, peaks, measured, uuid, rank, world, full):
                  "peak_source": f"{peaks['source']} HBM copy bandwidth"}
             if measured:
                 # tensor pipe: algorithmic flops over the measured MMA peak of the dtype the MMAs run in
-                # (BF16 features: kind::f16 forward, kind::tf32 backward; FP32 features: kind::tf32)
+                # (kind::f16, but kind::tf32 in the backward projection of BF16 features)
                 tflops = work[kind]["flops"] / (per_step_ms / 1000.0) / 1e12
-                mma = "bf16_mma" if (kind == "project" and wl.feat_dtype == "bf16") else "tf32_mma"
+                mma = "tf32_mma" if (kind == "project_bwd" and wl.feat_dtype == "bf16") else "bf16_mma"
                 r["tensor"] = {"achieved_tflops": tflops, "peak_tflops": measured[mma], "peak": mma,
                                "frac": tflops / measured[mma]}
             return r
         if kind == "adj_gemm":
             # tensor cores when the knob says so, or by the library's built-in choice
-            # (fmap_options.adjoint_kernel = 0): at least two 128-column dA_x tiles per SM
+            # (fmap_options.adjoint_kernel = 0): flops per K-block of the longest pair's chain
             ach = work[kind]["flops"] / (per_step_ms / 1000.0) / 1e12
             ak = fixed_tuning.get("adjoint_kernel", 0)
-            if ak == 1 or (ak == 0 and work[kind]["da_tiles"] >= 2 * SM_COUNT):
+            if ak == 1 or (ak == 0 and work[kind]["flops"] > 88e6 * work[kind]["blocks"]):
                 pk = measured["tf32_mma"] / 3.0 if measured else None
                 return {"kernel": kind, "bound": "tensor", "achieved": ach, "peak": pk, "unit": "TFLOP/s",
                         "frac": ach / pk if pk else None, "traffic": None,

@@ -426,14 +426,11 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
     P.bw_smem = fixed + out_staging + region;
   }
   if (P.tc_bwd32) {
-    // FP32 features: one CTA per SM over (shape, feature group, vertex chunk) items; a
-    // group is 64 features (32 when the basis needs more than 6 blocks of 32, so that the
-    // TF32 head and remainder images of dA^T plus two Phi stages fit), with its two
-    // images contiguous in the workspace. Items sorted by cost, dealt round-robin.
-    int kb_max = 1;
-    for (int s = 0; s < n_shapes; ++s)
-      if (P.shapes[s].dfeat) kb_max = std::max(kb_max, (P.shapes[s].k + 31) / 32);
-    const int nf_g = kb_max <= 6 ? 64 : 32;
+    // FP32 features: one CTA per SM over (shape, vertex chunk, feature group) items; a group is
+    // 64 features, whose image of dA^T thirds and four Phi tiles fit at any k. Items sorted by
+    // cost, dealt round-robin; the groups of a chunk stay neighbours, so that they run at the
+    // same time and its Phi is read from memory once.
+    const int nf_g = 64;
     int64_t bw_work = 0;
     for (int s = 0; s < n_shapes; ++s)
       if (P.shapes[s].dfeat) bw_work += P.shapes[s].n * (int64_t)((P.shapes[s].d + nf_g - 1) / nf_g);
@@ -445,22 +442,26 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
       const ShapeDev& sd = P.shapes[s];
       if (!sd.dfeat) continue;
       const int kb = (sd.k + 31) / 32;
+      const size_t g0 = P.bw_groups.size();
       for (int f0 = 0; f0 < sd.d; f0 += nf_g) {
         TcBwdGroup bg{};
         bg.shape = s; bg.f0 = f0; bg.nf = std::min(nf_g, sd.d - f0); bg.kb = kb;
         bg.img_off = cur;
-        cur = align_up(cur + 2 * (int64_t)kb * bg.nf * 32, kAlignFloats);
+        const int img = (kb + 1) / 2 * 3 * bg.nf * 32;      // floats
+        cur = align_up(cur + img, kAlignFloats);
         P.bw_groups.push_back(bg);
-        P.bw_max_img = std::max(P.bw_max_img, kb * bg.nf * 32);
-        P.bw_b_bytes = std::max<uint32_t>(P.bw_b_bytes, (uint32_t)(kb * bg.nf * 128));
-        for (int64_t v0 = 0; v0 < sd.n; v0 += bw_chunk) {
+        P.bw_max_img = std::max(P.bw_max_img, (kb + 1) / 2 * bg.nf * 8);
+        P.bw_b_bytes = std::max<uint32_t>(P.bw_b_bytes, (uint32_t)img * 4u);
+      }
+      for (int64_t v0 = 0; v0 < sd.n; v0 += bw_chunk)
+        for (size_t g = g0; g < P.bw_groups.size(); ++g) {
+          const TcBwdGroup& bg = P.bw_groups[g];
           TcBwdItem it{};
-          it.shape = s; it.f0 = f0; it.nf = bg.nf; it.kb = kb;
+          it.shape = s; it.f0 = bg.f0; it.nf = bg.nf; it.kb = kb;
           it.v0 = v0; it.v1 = std::min<int64_t>(sd.n, v0 + bw_chunk);
           it.img_off = bg.img_off;
           items.push_back(it);
         }
-      }
     }
     if (!items.empty()) {
       std::vector<int32_t> order(items.size());
@@ -483,9 +484,9 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
     }
     const int fixed = 1024 + 512;
     const int out_staging = 8 * 4096;   // FP32 dF staging of the eight epilogue warps
-    P.bw_stages = std::min(6, (kSmemBudget - fixed - out_staging - 2 * (int)P.bw_b_bytes) / 32768);
+    P.bw_stages = std::min(8, (kSmemBudget - fixed - out_staging - (int)P.bw_b_bytes) / 16384);
     if (!P.bw_items.empty() && P.bw_stages < 2) return FMAP_ERR_UNSUPPORTED;
-    P.bw_smem = fixed + out_staging + 2 * (int)P.bw_b_bytes + P.bw_stages * 32768;
+    P.bw_smem = fixed + out_staging + (int)P.bw_b_bytes + P.bw_stages * 16384;
   }
   const int64_t ws_bwd = std::max(cur, ws_fwd);
 
@@ -1094,8 +1095,8 @@ int32_t project_backward_impl(fmap_batch* b, const float* da, float* w, void* ws
   bp.cta_first = b->d_bw_cta_first;
   bp.stages = P.bw_stages;
   bp.b_bytes_max = P.bw_b_bytes;
-  // two accumulators: <= 64 columns each (FP32), or N = bw_max_nf rounded to a power of two
-  bp.tmem_cols = 128;
+  // two accumulators of N = bw_max_nf rounded to a power of two (FP32: of three sums, and operand slots)
+  bp.tmem_cols = 512;
   if (!P.tc_bwd32)
     for (bp.tmem_cols = 64; bp.tmem_cols < 2u * (uint32_t)P.bw_max_nf;) bp.tmem_cols <<= 1;
   bp.ws = w;

@@ -314,10 +314,11 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
   if (threadIdx.x == 0 && *abort_flag) atomicExch(P.err, (int)FMAP_ERR_TIMEOUT);
 }
 
-// A_s[n0 + n][f0 + f] = sum over the group's partials [n][f], in a fixed order: four thread groups
-// take every fourth partial, four loads in flight each, and their sums are added in order (one
-// thread adding every partial waits for one L2 round trip after another: one pair of n = 5000,
-// 76 partials per shape: 17 us against 11).
+// A_s[n0 + n][f0 + f] = sum over the group's partials [n][f], in a fixed order. From 16 partials four
+// thread groups take every fourth one, four loads in flight each, and their sums are added in order
+// (one thread adding every partial waits for one L2 round trip after another: one pair of n = 5000,
+// 76 partials per shape: 17 us against 11); below, a thread takes all of them (40 shapes of n = 1000,
+// k = 250, d = 512, 2 partials: 43 us in four groups, 24 so; 64 of n = 4000, k = 200, d = 256, 8: 38, 31).
 __global__ void __launch_bounds__(256) project_tc_reduce_kernel(const ShapeDev* shapes, const int64_t* parts,
                                                                 const TcRedGroup* groups, float* a_out, const float* ws) {
   __shared__ float4 red[3][64];
@@ -327,33 +328,39 @@ __global__ void __launch_bounds__(256) project_tc_reduce_kernel(const ShapeDev* 
   // partials are 256-byte aligned; float4 stores when the output buffer is 16-byte aligned)
   const int q4 = g.dspan >> 2, total = g.nk * q4;
   const bool vec = (reinterpret_cast<uintptr_t>(a_out) & 15) == 0;
-  const int sub = threadIdx.x >> 6, lane = threadIdx.x & 63;
-  for (int e0 = blockIdx.x * 64; e0 < total; e0 += gridDim.x * 64) {
+  float* out = a_out + s.a_off + (int64_t)g.n0 * s.d + g.f0;
+  const int subs = g.part_end - g.part_beg < 16 ? 1 : 4, per = 256 / subs;      // thread groups, elements of each
+  const int sub = threadIdx.x / per, lane = threadIdx.x - sub * per;
+  for (int e0 = blockIdx.x * per; e0 < total; e0 += gridDim.x * per) {
     const int e = e0 + lane;
     const int n = e / q4, f = (e - n * q4) * 4;
     const float* src = ws + (int64_t)n * g.stride + f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (e < total) {
-      for (int i = g.part_beg + sub; i < g.part_end; i += 16) {
+      for (int i = g.part_beg + sub; i < g.part_end; i += 4 * subs) {
         float4 u[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          u[j] = i + 4 * j < g.part_end ? *reinterpret_cast<const float4*>(src + __ldg(parts + i + 4 * j))
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+          u[j] = i + subs * j < g.part_end ? *reinterpret_cast<const float4*>(src + __ldg(parts + i + subs * j))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int j = 0; j < 4; ++j) { acc.x += u[j].x; acc.y += u[j].y; acc.z += u[j].z; acc.w += u[j].w; }
       }
     }
-    __syncthreads();                   // (the previous round's sums have been read)
-    if (sub > 0) red[sub - 1][lane] = acc;
-    __syncthreads();
-    if (sub == 0 && e < total) {
+    if (subs > 1) {
+      __syncthreads();                 // (the previous round's sums have been read)
+      if (sub > 0) red[sub - 1][lane] = acc;
+      __syncthreads();
+      if (sub == 0) {
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const float4 u = red[j][lane];
-        acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
+        for (int j = 0; j < 3; ++j) {
+          const float4 u = red[j][lane];
+          acc.x += u.x; acc.y += u.y; acc.z += u.z; acc.w += u.w;
+        }
       }
-      float* o = a_out + s.a_off + (int64_t)(g.n0 + n) * s.d + g.f0 + f;
+    }
+    if (sub == 0 && e < total) {
+      float* o = out + (int64_t)n * s.d + f;
       if (vec) {
         *reinterpret_cast<float4*>(o) = acc;
       } else {

@@ -48,18 +48,6 @@ constexpr int kStepV = 16;                        // vertices per K-step (one sl
 constexpr uint32_t kBoxBytes = kStageV * 128;     // one TMA box: 32 vertices x 32 FP32 (features or basis)
 constexpr uint32_t kColBytes = kStepV * 128;      // 16 vertices x 64 basis functions of one third
 
-// (a, b) -> heads, middles and tails, each pair packed low = a, high = b.
-__device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
-  a -= __uint_as_float(hi << 16); b -= __uint_as_float(hi & 0xffff0000u);
-  const __nv_bfloat162 m = __floats2bfloat162_rn(a, b);
-  mid = *reinterpret_cast<const uint32_t*>(&m);
-  a -= __uint_as_float(mid << 16); b -= __uint_as_float(mid & 0xffff0000u);
-  const __nv_bfloat162 l = __floats2bfloat162_rn(a, b);
-  lo = *reinterpret_cast<const uint32_t*>(&l);
-}
-
 // The whole warp waits and goes on, or gives up, together.
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
   return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort));
@@ -250,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
           }
           uint32_t h[4], md[4], l[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) split3(x[2 * i], x[2 * i + 1], h[i], md[i], l[i]);
+          for (int i = 0; i < 4; ++i) tc::split3(x[2 * i], x[2 * i + 1], h[i], md[i], l[i]);
           if (!warp_wait(&part_empty[slot], slot_phase ^ 1, abort_flag)) goto done;
           tc::tc_fence_after();
           const uint32_t a = lane_base + 512u - (uint32_t)((slot * item.fg + m + 1) * kTc32SlotCols) + c0 * 4;
@@ -259,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
           tc::tmem_st4(a + 16, l);
           if (two) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) split3(x[8 + 2 * i], x[9 + 2 * i], h[i], md[i], l[i]);
+            for (int i = 0; i < 4; ++i) tc::split3(x[8 + 2 * i], x[9 + 2 * i], h[i], md[i], l[i]);
             tc::tmem_st4(a + 4, h);
             tc::tmem_st4(a + 12, md);
             tc::tmem_st4(a + 20, l);
@@ -359,10 +347,10 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
               if (g0 + e >= ng) break;
               const float4 p = swap ? y[e] : x[e], q = swap ? x[e] : y[e];
               uint4 h, md, l;
-              split3(p.x * mv, p.y * mv, h.x, md.x, l.x);
-              split3(p.z * mv, p.w * mv, h.y, md.y, l.y);
-              split3(q.x * mv, q.y * mv, h.z, md.z, l.z);
-              split3(q.z * mv, q.w * mv, h.w, md.w, l.w);
+              tc::split3(p.x * mv, p.y * mv, h.x, md.x, l.x);
+              tc::split3(p.z * mv, p.w * mv, h.y, md.y, l.y);
+              tc::split3(q.x * mv, q.y * mv, h.z, md.z, l.z);
+              tc::split3(q.z * mv, q.w * mv, h.w, md.w, l.w);
               if (g0 + e == 0 && !warp_wait(&part_empty[slot], slot_phase ^ 1, abort_flag)) goto done;
               if (on[e]) {
                 *reinterpret_cast<uint4*>(out + (g0 + e) * kColBytes + dst[0]) = h;
