@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kGfThreads, 1) gradfeat_kernel(GfParams P) {
       const int quarter = warp & 3;
       const int r = quarter * 32 + lane;
       const int64_t v = tile * kGfTileV + r;
-      const bool ok = tc::mbar_wait(acc_full, aphase, abort_flag);
+      const bool ok = tc::warp_wait(acc_full, aphase, abort_flag);
       aphase ^= 1;
       tc::tc_fence_after();
       for (int j = warp >> 2; ok && j < dim / 16; j += kGfGatherWarps / 4) {

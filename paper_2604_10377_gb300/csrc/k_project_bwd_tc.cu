@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_bwd_tc_kernel(TcBwdParams
         // the row's mass, loaded a tile ahead
         const float m = m_next;
         m_next = v + 2 * kTileV < item.v1 ? __ldg(s.mass + v + 2 * kTileV) : 0.f;
-        if (!tc::mbar_wait(&acc_full[buf], acc_phase[buf], abort_flag)) goto epi_done;
+        if (!tc::warp_wait(&acc_full[buf], acc_phase[buf], abort_flag)) goto epi_done;
         tc::tc_fence_after();
         const int rows = (int)(item.v1 - vrow0 < 32 ? item.v1 - vrow0 : 32);   // (may be negative)
         __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(s.dfeat) + vrow0 * s.ld_feat + item.f0;

@@ -42,11 +42,6 @@ constexpr int kTileV = 128;                          // vertices per output tile
 constexpr uint32_t kAStageBytes = kTileV * 128;      // 128 rows x 32 FP32
 constexpr uint32_t kOutWarpBytes = 32 * 128;         // 32 rows x 32 FP32: one TMA store box per epilogue warp
 
-// The whole warp waits and goes on, or gives up, together.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort));
-}
-
 __global__ void __launch_bounds__(kThreads, 1) project_bwd_tc32_kernel(TcBwdParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -142,7 +137,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_bwd_tc32_kernel(TcBwdPara
     for (int it = it_beg; it < it_end && ok; ++it) {
       const TcBwdItem item = P.items[it];
       const int steps = (P.shapes[item.shape].k + 15) / 16;
-      if (!warp_wait(b_full, bphase, abort_flag)) break;
+      if (!tc::warp_wait(b_full, bphase, abort_flag)) break;
       bphase ^= 1;
       tc::tc_fence_after();
       const uint32_t nf = (uint32_t)item.nf;
@@ -150,13 +145,13 @@ __global__ void __launch_bounds__(kThreads, 1) project_bwd_tc32_kernel(TcBwdPara
       const uint32_t i3 = tc::idesc_bf16_f32(128, 3 * nf, 0, 0);
       const int ntiles = (int)((item.v1 - item.v0 + kTileV - 1) / kTileV);
       for (int t = 0; t < ntiles && ok; ++t) {
-        if (!warp_wait(&acc_empty[buf], acc_phase[buf] ^ 1, abort_flag)) { ok = false; break; }
+        if (!tc::warp_wait(&acc_empty[buf], acc_phase[buf] ^ 1, abort_flag)) { ok = false; break; }
         tc::tc_fence_after();
         const uint32_t d = tmem_base + (uint32_t)(buf * kAccCols);
         for (int kb = 0; kb < item.kb; ++kb) {
           const uint64_t b = b0 + (uint64_t)((uint32_t)(kb >> 1) * 3u * nf * 8u + (uint32_t)(kb & 1) * 4u);
           const uint32_t a = tmem_base + (uint32_t)(kBufs * kAccCols) + slot * kSlotCols;
-          if (!warp_wait(&slot_full[slot], slot_phase, abort_flag)) { ok = false; break; }
+          if (!tc::warp_wait(&slot_full[slot], slot_phase, abort_flag)) { ok = false; break; }
           tc::tc_fence_after();
           if (lead) {
 #pragma unroll
@@ -191,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_bwd_tc32_kernel(TcBwdPara
       const uint32_t end = block + (uint32_t)((item.v1 - item.v0 + kTileV - 1) / kTileV) * (uint32_t)item.kb;
       for (uint32_t g = block + ((block + (uint32_t)set) & 1); g < end; g += 2) {
         const uint32_t a = a0 + slot * kSlotCols;
-        if (!warp_wait(&a_full[stage], phase, abort_flag)) goto conv_done;
+        if (!tc::warp_wait(&a_full[stage], phase, abort_flag)) goto conv_done;
         const uint8_t* src = sA + (size_t)stage * kAStageBytes + row * 128;
         uint32_t hi[8], mid[8], lo[8];
 #pragma unroll
@@ -200,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_bwd_tc32_kernel(TcBwdPara
           tc::split3(x.x, x.y, hi[2 * z], mid[2 * z], lo[2 * z]);
           tc::split3(x.z, x.w, hi[2 * z + 1], mid[2 * z + 1], lo[2 * z + 1]);
         }
-        if (!warp_wait(&slot_empty[slot], slot_phase ^ 1, abort_flag)) goto conv_done;
+        if (!tc::warp_wait(&slot_empty[slot], slot_phase ^ 1, abort_flag)) goto conv_done;
         tc::tc_fence_after();
         tc::tmem_st8(a, hi);
         tc::tmem_st8(a + 8, mid);
@@ -232,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_bwd_tc32_kernel(TcBwdPara
         const int64_t vrow0 = item.v0 + (int64_t)t * kTileV + quarter * 32;
         const int64_t v = vrow0 + lane;
         const float m = v < item.v1 ? __ldg(s.mass + v) : 0.f;
-        if (!tc::mbar_wait(&acc_full[buf], acc_phase[buf], abort_flag)) goto epi_done;
+        if (!tc::warp_wait(&acc_full[buf], acc_phase[buf], abort_flag)) goto epi_done;
         tc::tc_fence_after();
         // 32 features per warp, 128-byte rows with the 128-byte swizzle (conflict-free, and half as
         // many box rows as 16 features would make: a TMA store takes about 6 cycles per row)

@@ -50,11 +50,6 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint3
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// The whole warp waits and goes on, or gives up, together.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort));
-}
-
 // The MMAs of one segment. kV: vertices per stage; kFg: feature groups (0: item.fg); kMerged: tc_merged. One
 // lane issues them and the time per MMA counts at small k, so the descriptors are computed ahead of the waits.
 template <int kV, int kFg, bool kMerged>
@@ -70,7 +65,7 @@ __device__ __forceinline__ bool issue(const TcProjParams& P, const TcItem& item,
   for (int st = 0; st < nst; ++st) {
     const uint64_t ad = tc::smem_desc(tc::smem_u32(sF + (size_t)stage * P.f_stage_bytes), kV * 128, 1024, tc::kLayoutSW128);
     const uint64_t bd = tc::smem_desc(tc::smem_u32(sP + (size_t)stage * P.p_stage_bytes), 16, 1024, tc::kLayoutSW128);
-    if (!warp_wait(&full_f[stage], phase, abort) || !warp_wait(&full_p[stage], phase, abort)) return false;
+    if (!tc::warp_wait(&full_f[stage], phase, abort) || !tc::warp_wait(&full_p[stage], phase, abort)) return false;
     tc::tc_fence_after();
 #pragma unroll
     for (int kk = 0; kk < kV / 16; ++kk) {
@@ -148,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
           tc::prefetch_tmap(mmap);
         }
         for (int st = 0; st < nst; ++st) {
-          if (!warp_wait(&empty[stage], phase ^ 1, abort_flag)) goto producer_done;
+          if (!tc::warp_wait(&empty[stage], phase ^ 1, abort_flag)) goto producer_done;
           if (lane == 0) tc::mbar_arrive_expect_tx(&full_f[stage], bytes);
           __syncwarp();
           const int y = (int)(item.v0 + (int64_t)st * kStageV);
@@ -180,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
     uint32_t stage = 0, phase = 0, acc_phase = 0;
     for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
       const TcItem item = P.items[it];
-      if (!warp_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
+      if (!tc::warp_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
       tc::tc_fence_after();
       const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
       bool ok;
@@ -203,14 +198,17 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
     const int cw = warp - 2;
     const int qs = lane & 7, csub = lane >> 3;
     uint32_t stage = 0, phase = 0, acc_phase = 0;
+    // no wait of this warp has given up. The converters meet in a barrier per stage, so a warp whose wait
+    // gave up goes through the remaining stages and their barriers without working (every other wait
+    // then ends at once) instead of leaving the others there
+    bool ok = true;
     for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
       const TcItem item = P.items[it];
       const ShapeDev s = P.shapes[item.shape];
-      const int k = s.k;
       const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
       const int kb = (item.npad + 31) / 32;
       for (int st = 0; st < nst; ++st) {
-        if (!tc::mbar_wait(&full_f[stage], phase, abort_flag)) goto conv_done;
+        ok = ok && tc::warp_wait(&full_f[stage], phase, abort_flag);
         uint8_t* tile = sP + (size_t)stage * P.p_stage_bytes;
         const float* mst = sM + (size_t)stage * kStageV;
         const int64_t vbase = item.v0 + (int64_t)st * kStageV;
@@ -264,16 +262,15 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
             }
           }
         }
-        (void)k;
         tc::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&full_p[stage]);
         if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
       }
       // epilogue: accumulators -> this item's partial A (k x stride, row-major)
-      if (!tc::mbar_wait(acc_full, acc_phase, abort_flag)) goto conv_done;
+      ok = ok && tc::warp_wait(acc_full, acc_phase, abort_flag);
       tc::tc_fence_after();
-      {
+      if (ok) {
         const int quarter = warp & 3, half = cw >> 2;
         const int stride = item.fg * 128;
         float* part = P.ws + item.part_off;
@@ -306,7 +303,6 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
       if (lane == 0) tc::mbar_arrive(acc_empty);
       acc_phase ^= 1;
     }
-  conv_done:;
   }
 
   __syncthreads();

@@ -48,11 +48,6 @@ constexpr int kStepV = 16;                        // vertices per K-step (one sl
 constexpr uint32_t kBoxBytes = kStageV * 128;     // one TMA box: 32 vertices x 32 FP32 (features or basis)
 constexpr uint32_t kColBytes = kStepV * 128;      // 16 vertices x 64 basis functions of one third
 
-// The whole warp waits and goes on, or gives up, together.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort));
-}
-
 // The MMAs of one segment of kFg feature groups and kAccs accumulators each. One thread issues them,
 // and at small k the time it takes per MMA counts: everything but the waits is computed beforehand.
 template <int kFg, int kAccs>
@@ -70,7 +65,7 @@ __device__ __forceinline__ bool issue(const TcProjParams& P, const TcItem& item,
   for (int st = 0; st < nst; ++st) {
 #pragma unroll
     for (int q = 0; q < kTc32Slots; ++q) {
-      if (!warp_wait(&part_full[q], phase, abort)) return false;
+      if (!tc::warp_wait(&part_full[q], phase, abort)) return false;
       tc::tc_fence_after();
       const uint32_t on = st == 0 && q == 0 ? 0u : 1u;
 #pragma unroll
@@ -159,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
           tc::prefetch_tmap(mmap);
         }
         for (int st = 0; st < nst; ++st) {
-          if (!warp_wait(&empty[stage], phase ^ 1, abort_flag)) goto producer_done;
+          if (!tc::warp_wait(&empty[stage], phase ^ 1, abort_flag)) goto producer_done;
           if (lane == 0) tc::mbar_arrive_expect_tx(&full[stage], bytes);
           __syncwarp();
           const int y = (int)(item.v0 + (int64_t)st * kStageV);
@@ -188,7 +183,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
       uint32_t phase = 0, acc_phase = 0;
       for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
         const TcItem item = P.items[it];
-        if (!warp_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
+        if (!tc::warp_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
         tc::tc_fence_after();
         const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
         const int accs = tc32_accs(item.fg, item.npad);
@@ -225,7 +220,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
       const int m = two ? set : 0;
       const uint32_t c0 = two ? 0u : (uint32_t)set;
       for (int st = 0; st < nst; ++st) {
-        if (!warp_wait(&full[stage], phase, abort_flag)) goto done;
+        if (!tc::warp_wait(&full[stage], phase, abort_flag)) goto done;
         const uint8_t* tile = sF + (size_t)stage * P.f_stage_bytes + (m * 4 + quarter) * kBoxBytes + c0 * 1024;
 #pragma unroll
         for (int step = 0; step < kStageV / kStepV; ++step) {
@@ -239,7 +234,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
           uint32_t h[4], md[4], l[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) tc::split3(x[2 * i], x[2 * i + 1], h[i], md[i], l[i]);
-          if (!warp_wait(&part_empty[slot], slot_phase ^ 1, abort_flag)) goto done;
+          if (!tc::warp_wait(&part_empty[slot], slot_phase ^ 1, abort_flag)) goto done;
           tc::tc_fence_after();
           const uint32_t a = lane_base + 512u - (uint32_t)((slot * item.fg + m + 1) * kTc32SlotCols) + c0 * 4;
           tc::tmem_st4(a, h);
@@ -265,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
         if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
       }
       // accumulators -> this item's partial A (nk x stride, row-major)
-      if (!warp_wait(acc_full, acc_phase, abort_flag)) goto done;
+      if (!tc::warp_wait(acc_full, acc_phase, abort_flag)) goto done;
       tc::tc_fence_after();
       {
         const int accs = tc32_accs(item.fg, item.npad);
@@ -322,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
         dst[p] = (uint32_t)(ci >> 3) * kColBytes + (uint32_t)v * 128u + ((uint32_t)((ci ^ v) & 7) << 4);
       }
       for (int st = 0; st < nst; ++st) {
-        if (!warp_wait(&full[stage], phase, abort_flag)) goto done;
+        if (!tc::warp_wait(&full[stage], phase, abort_flag)) goto done;
 #pragma unroll
         for (int step = 0; step < kStageV / kStepV; ++step) {
           const uint8_t* phi = sP + (size_t)stage * P.p_stage_bytes + step * kStepV * 128;
@@ -351,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc32_kernel(TcProjParams 
               tc::split3(p.z * mv, p.w * mv, h.y, md.y, l.y);
               tc::split3(q.x * mv, q.y * mv, h.z, md.z, l.z);
               tc::split3(q.z * mv, q.w * mv, h.w, md.w, l.w);
-              if (g0 + e == 0 && !warp_wait(&part_empty[slot], slot_phase ^ 1, abort_flag)) goto done;
+              if (g0 + e == 0 && !tc::warp_wait(&part_empty[slot], slot_phase ^ 1, abort_flag)) goto done;
               if (on[e]) {
                 *reinterpret_cast<uint4*>(out + (g0 + e) * kColBytes + dst[0]) = h;
                 *reinterpret_cast<uint4*>(out + (g0 + e) * kColBytes + dst[1]) = md;
