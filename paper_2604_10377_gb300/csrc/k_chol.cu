@@ -775,8 +775,10 @@ __device__ __forceinline__ void row_update(float (&s)[8], const float (&x)[8], c
 }
 
 // Cholesky factor of the 8 x 8 block d (lower part) in registers, r[j] = 1 / L_jj. kSafe:
-// reciprocal square roots that also take subnormal pivots, and a check of every pivot;
-// without it a bad or subnormal pivot leaves a value that is not finite and positive in r[7].
+// reciprocal square roots that also take subnormal pivots, and a check of every pivot.
+// Without it the caller tests r: a pivot that is negative, zero, subnormal or not a number spreads
+// through the updates and leaves a value that is not finite and positive in r[7]; an infinite one
+// leaves its own r[j] = 0 and the columns after it untouched.
 template <bool kSafe>
 __device__ __forceinline__ bool factor8(float (&d)[8][8], float (&r)[8]) {
   bool ok = true;
@@ -928,7 +930,8 @@ __device__ __forceinline__ void factor_registers(float* S, float* linv, float* p
       float d[8][8], r[8];
       load_lower8(dbuf, 8, d);
       factor8<false>(d, r);
-      if (!(r[7] > 0.f && r[7] < INFINITY)) {
+      const float rmin = fminf(fminf(fminf(r[0], r[1]), fminf(r[2], r[3])), fminf(fminf(r[4], r[5]), r[6]));
+      if (!(r[7] > 0.f && r[7] < INFINITY && rmin > 0.f)) {
         load_lower8(dbuf, 8, d);
         if (!factor8<true>(d, r)) *s_bad = 1;
       }
