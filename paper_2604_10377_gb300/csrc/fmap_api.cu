@@ -93,7 +93,6 @@ struct Plan {
   std::vector<TcRedGroup> tc_groups;
   std::vector<int64_t> tc_parts;       // offsets of the partials, group after group
   int64_t tc_max_group_elems = 0;
-  int tc_smem = 0;                     // the largest dynamic shared memory of the launches
   // tensor-core backward projection
   std::vector<TcBwdItem> bw_items;
   std::vector<int32_t> bw_cta_first;   // bwd_ctas + 1 (FP32) or bwd_ctas / 2 + 1 (BF16) boundaries
@@ -323,7 +322,6 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
       L.stages = std::min(opt.proj_max_stages ? opt.proj_max_stages : 6, (kSmemBudget - fixed) / per_stage);
       if (L.stages < 2) return FMAP_ERR_UNSUPPORTED;
       L.smem = fixed + L.stages * per_stage;
-      P.tc_smem = std::max(P.tc_smem, L.smem);
       P.tc_launches.push_back(L);
     }
   }
@@ -844,14 +842,15 @@ int32_t fmap_batch_create(fmap_ctx* ctx, const fmap_shape_desc* shapes, int32_t 
     put(o_bo, P.bw_cta_first.data(), P.bw_cta_first.size() * sizeof(int32_t));
     put(o_bg, P.bw_groups.data(), P.bw_groups.size() * sizeof(TcBwdGroup));
     if (!P.bw_items.empty()) {
-      e = P.tc_bwd32 ? project_bwd_tc32_set_smem(P.bw_smem) : project_bwd_tc_set_smem(P.bw_smem);
+      e = P.tc_bwd32 ? project_bwd_tc32_set_smem(kSmemBudget) : project_bwd_tc_set_smem(kSmemBudget);
       if (e != cudaSuccess) { cudaFree(b->dev_mem); delete b; return cuda_fail(e, "cudaFuncSetAttribute(project bwd)"); }
     }
     put(o_ti, P.tc_items.data(), P.tc_items.size() * sizeof(TcItem));
     put(o_to, P.tc_cta_first.data(), P.tc_cta_first.size() * sizeof(int32_t));
     put(o_tg, P.tc_groups.data(), P.tc_groups.size() * sizeof(TcRedGroup));
     put(o_tp, P.tc_parts.data(), P.tc_parts.size() * sizeof(int64_t));
-    e = P.tc32 ? project_tc32_set_smem(P.tc_smem) : project_tc_set_smem(P.tc_smem);
+    // (the limits belong to the kernels, not to a batch: every batch sets the same one)
+    e = P.tc32 ? project_tc32_set_smem(kSmemBudget) : project_tc_set_smem(kSmemBudget);
     if (e != cudaSuccess) { cudaFree(b->dev_mem); delete b; return cuda_fail(e, "cudaFuncSetAttribute(project)"); }
   }
   e = cudaMemcpy(b->dev_mem, host.data(), (size_t)total, cudaMemcpyHostToDevice);
