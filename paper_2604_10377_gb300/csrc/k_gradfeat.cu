@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kGfThreads, 1) gradfeat_kernel(GfParams P) {
     const int gr = warp * 8 + sub;                       // its row of the tile
     const char* x_lane = reinterpret_cast<const char*>(P.x_in) + 16 * cl;
     const uint64_t ldb = (uint64_t)P.ld_in * 4u;
+    const uint32_t n_cols = (uint32_t)(P.n_in < ((int64_t)1 << 31) ? P.n_in : (int64_t)1 << 31);
     // CSR offsets of the vertex in `tile` (length 0 outside the operator)
     auto meta = [&](int64_t tile, int64_t& e0, int& len) {
       const int64_t v = tile * kGfTileV + gr;
@@ -196,6 +197,7 @@ __global__ void __launch_bounds__(kGfThreads, 1) gradfeat_kernel(GfParams P) {
     };
     // entries q .. q+7 of a row (column -1: none); a column outside X is reported and skipped
     auto entries = [&](int64_t e0, int len, int q, int32_t (&c)[8], float2 (&g)[8]) {
+      bool bad = false;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         c[u] = -1;
@@ -203,11 +205,17 @@ __global__ void __launch_bounds__(kGfThreads, 1) gradfeat_kernel(GfParams P) {
         if (q + u < len) {
           const int32_t cc = __ldg(P.col_idx + e0 + q + u);
           g[u] = __ldg(P.vals + e0 + q + u);
-          if (cc >= 0 && cc < P.n_in)
+          if ((uint32_t)cc < n_cols)
             c[u] = cc;
           else
-            *bad_index = 1;
+            bad = true;
         }
+      }
+      if (bad) {             // (the values of skipped entries stay out too: they need not be finite)
+        *bad_index = 1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (c[u] < 0) g[u] = make_float2(0.f, 0.f);
       }
     };
     // (ax, ay) += the entries' values times four channels of their rows of X, 64 j bytes on
