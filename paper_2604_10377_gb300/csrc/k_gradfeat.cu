@@ -364,7 +364,9 @@ extern "C" FMAP_API int32_t fmap_gradient_features(int64_t n, const int64_t* row
     return FMAP_ERR_CUDA;
   const size_t smem = gf_smem_bytes(dim);
   auto* kernel = ld_in >= ((int64_t)1 << 30) ? gradfeat_kernel<true> : gradfeat_kernel<false>;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  // the limit belongs to the kernel, which other threads launch too: the same for every D
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gf_smem_bytes(kGfMaxDim)) !=
+      cudaSuccess)
     return FMAP_ERR_CUDA;
   if (cudaMemsetAsync(status, 0, sizeof(int32_t), st) != cudaSuccess) return FMAP_ERR_CUDA;
   float* img = static_cast<float*>(ws);
