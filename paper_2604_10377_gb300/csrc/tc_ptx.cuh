@@ -350,8 +350,8 @@ __device__ __forceinline__ float tf32_rna(float x) {
 // (a, b) -> the BF16 heads, middles and tails (8 bits each, rounded to nearest) whose sums they are
 // exactly, each pair packed low = a, high = b.
 __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
+  // (finite numbers above the largest BF16 keep a finite head)
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(b), "f"(a));
   a -= __uint_as_float(hi << 16); b -= __uint_as_float(hi & 0xffff0000u);
   const __nv_bfloat162 m = __floats2bfloat162_rn(a, b);
   mid = *reinterpret_cast<const uint32_t*>(&m);
