@@ -200,7 +200,6 @@ def algorithmic_work(wl, ir_steps, saved_k_max):
     bwd_bytes = sum(s.n * (4 * s.k + 4 + fsz * s.d) + 4 * s.k * s.d for s in wl.shapes)
     solve_flops, adj_flops, loss_flops, gemm_flops = 0.0, 0.0, 0.0, 0.0
     solve_bytes, adj_bytes = 0, 0
-    gemm_blocks = 0
     for p in wl.pairs:
         # C is ky x k: ky row systems of size k (square maps: ky == k)
         k, ky = wl.shapes[p.x].k, wl.shapes[p.y].k
@@ -213,13 +212,12 @@ def algorithmic_work(wl, ir_steps, saved_k_max):
         # adjoint GEMMs: W = Gamma^T C + C^T Gamma, dA_y = Gamma A_x, dA_x = Gamma^T A_y - W A_x
         d = wl.shapes[p.x].d
         gemm_flops += 4.0 * k * k * ky + 2.0 * ky * k * d + 2.0 * k * (ky + k) * d
-        gemm_blocks = max(gemm_blocks, -(-max(2 * ky, k) // 32) + -(-(k + ky) // 32))
         # G, R and C move once each, saved factors written (forward) / read (adjoint)
         solve_bytes += 4 * (k * k + 2 * ky * k) + fac
         adj_bytes += 4 * 2 * ky * k + fac
     return dict(project=dict(bytes=proj_bytes, flops=proj_flops), project_bwd=dict(bytes=bwd_bytes, flops=proj_flops),
                 solve=dict(flops=solve_flops, bytes=solve_bytes), adj_solve=dict(flops=adj_flops, bytes=adj_bytes),
-                loss=dict(flops=loss_flops), adj_gemm=dict(flops=gemm_flops, blocks=gemm_blocks))
+                loss=dict(flops=loss_flops), adj_gemm=dict(flops=gemm_flops))
 
 
 # ---------------------------------------------------------------- oracle timing
@@ -629,18 +627,14 @@ def bench_workload(wid, args, dev, peaks, measured, uuid, rank, world, full):
                                "frac": tflops / measured[mma]}
             return r
         if kind == "adj_gemm":
-            # tensor cores when the knob says so, or by the library's built-in choice
-            # (fmap_options.adjoint_kernel = 0): flops per K-block of the longest pair's chain
+            # on the FP32 FMA tiles or the tensor cores, by the library's choice for the batch
+            # (fmap_options.adjoint_kernel = 0) or the knob's: the rate against both peaks
             ach = work[kind]["flops"] / (per_step_ms / 1000.0) / 1e12
-            ak = fixed_tuning.get("adjoint_kernel", 0)
-            if ak == 1 or (ak == 0 and work[kind]["flops"] > 88e6 * work[kind]["blocks"]):
-                pk = measured["tf32_mma"] / 3.0 if measured else None
-                return {"kernel": kind, "bound": "tensor", "achieved": ach, "peak": pk, "unit": "TFLOP/s",
-                        "frac": ach / pk if pk else None, "traffic": None,
-                        "peak_source": "measured TF32 MMA peak / 3 (three TF32 passes per FP32-class product)"
-                        if pk else "TF32 peak not measured (--no-peaks)"}
-            return {"kernel": kind, "bound": "alu", "achieved": ach, "peak": fp32_peak_tflops, "unit": "TFLOP/s",
-                    "frac": ach / fp32_peak_tflops, "traffic": None, "peak_source": fp32_peak_source}
+            pk = measured["tf32_mma"] / 3.0 if measured else None
+            return {"kernel": kind, "bound": "tensor or alu", "achieved": ach, "peak": pk, "unit": "TFLOP/s",
+                    "frac": ach / pk if pk else None, "frac_of_fp32": ach / fp32_peak_tflops, "traffic": None,
+                    "peak_source": "measured TF32 MMA peak / 3 (three TF32 passes per FP32-class product)"
+                    if pk else "TF32 peak not measured (--no-peaks)"}
         flops = work.get(kind, {}).get("flops")
         if flops is None:
             return {"kernel": kind, "bound": "alu", "achieved": None, "peak": fp32_peak_tflops, "unit": "TFLOP/s",

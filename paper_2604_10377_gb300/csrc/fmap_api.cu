@@ -102,6 +102,7 @@ struct Plan {
   // tensor-core adjoint GEMMs (built when the batch is created: the SM count sets the tiles)
   AdjTcPlan adj;
   AdjTcPlan loss_tc;        // the training loss's GEMMs on the same kernel (E, then dL/dC)
+  int adj_tile = 32, loss_tile = 32;   // and the tiles of both on the CUDA cores
   bool row_grads = false;   // some pair has per-row lambda gradients to write
   fmap_sizes sizes{};
 };
@@ -713,10 +714,12 @@ int32_t fmap_batch_create(fmap_ctx* ctx, const fmap_shape_desc* shapes, int32_t 
     cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, ctx->device);
     b->sm_count = dev_sms > 0 ? dev_sms : kTcCtas;
   }
+  std::vector<int3> pk(P.pairs.size());
+  for (size_t p = 0; p < P.pairs.size(); ++p)
+    pk[p] = make_int3(P.pairs[p].k, P.shapes[P.pairs[p].y].k, P.pairs[p].d);
+  P.adj_tile = adjoint_simt_choice(pk).tile;
+  P.loss_tile = loss_simt_choice(pk).tile;
   if (ctx->opt.adjoint_kernel != 2 && n_pairs > 0) {
-    std::vector<int3> pk(P.pairs.size());
-    for (size_t p = 0; p < P.pairs.size(); ++p)
-      pk[p] = make_int3(P.pairs[p].k, P.shapes[P.pairs[p].y].k, P.pairs[p].d);
     P.adj.stages = ctx->opt.adjoint_stages;
     P.adj.features = ctx->opt.adjoint_features;
     adjoint_tc_plan(pk, b->sm_count, P.adj);
@@ -1059,10 +1062,10 @@ int32_t adjoint_impl(fmap_batch* b, const float* d_c, const float* a, const floa
   {
     TimedScope ts(b, FMAP_KIND_ADJ_GEMM, st);
     const int ak = b->plan.opt.adjoint_kernel;
-    const bool simt = ak == 2 || (ak == 0 && !b->plan.adj.tensor_cores);
+    const bool tc = ak == 1 || (ak == 0 && b->plan.adj.tensor_cores);
     e = launch_adjoint_gemms(b->dev, b->plan.max_k, b->plan.max_d, a, c, d_mask, d_lambda, b->plan.row_grads, w,
-                             simt, st);
-    if (e == cudaSuccess && !simt) e = launch_adjoint_tc(b->dev, b->d_adj_items, b->plan.adj, a, c, w, st);
+                             tc ? 0 : b->plan.adj_tile, st);
+    if (e == cudaSuccess && tc) e = launch_adjoint_tc(b->dev, b->d_adj_items, b->plan.adj, a, c, w, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "adjoint gemms");
   {
@@ -1196,7 +1199,7 @@ int32_t fmap_loss_orth(fmap_batch* b, const float* c, const float* c_gt, float* 
     e = tc ? launch_loss_tc(b->dev, b->d_loss_items, b->plan.loss_tc, c, c_gt, loss, d_c, w, w + b->plan.loss_part_off,
                             static_cast<cudaStream_t>(stream))
            : launch_loss_orth(b->dev, b->plan.max_k, c, c_gt, loss, d_c, w, w + b->plan.loss_part_off,
-                              static_cast<cudaStream_t>(stream));
+                              b->plan.loss_tile, static_cast<cudaStream_t>(stream));
   }
   if (e != cudaSuccess) return cuda_fail(e, "loss");
   return FMAP_OK;

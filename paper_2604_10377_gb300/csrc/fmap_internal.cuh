@@ -213,10 +213,10 @@ cudaError_t launch_solve(const BatchDev& b, const SolveGroup& g, const int2* sys
                          const float* rhs_flat, float* out_flat, float* saved_rw, int32_t* status,
                          float* ws, cudaStream_t st);
 // The mask and lambda gradients (when d_mask / d_lambda are given, or a pair has per-row
-// lambda outputs: row_grads) and, with simt, W and the dA contributions on the CUDA cores
-// (FP32 FMA tiles)
+// lambda outputs: row_grads) and, with simt_tile 32 or 64, W and the dA contributions on the CUDA
+// cores (FP32 FMA tiles of that edge)
 cudaError_t launch_adjoint_gemms(const BatchDev& b, int max_k, int max_d, const float* a, const float* c,
-                                 float* d_mask, float* d_lambda, bool row_grads, float* ws, bool simt,
+                                 float* d_mask, float* d_lambda, bool row_grads, float* ws, int simt_tile,
                                  cudaStream_t st);
 
 // One CTA of the tensor-core adjoint GEMMs: output rows r0 .. r0+127 and columns f0 .. f0+NT-1
@@ -238,7 +238,15 @@ cudaError_t launch_adjoint_tc(const BatchDev& b, const AdjItem* items, const Adj
 cudaError_t adjoint_tc_set_smem();
 cudaError_t launch_gather_da(const BatchDev& b, int max_kd, float* d_a, const float* ws, cudaStream_t st);
 cudaError_t launch_loss_orth(const BatchDev& b, int max_k, const float* c, const float* c_gt, float* loss,
-                             float* d_c, float* ws, float* partial, cudaStream_t st);
+                             float* d_c, float* ws, float* partial, int simt_tile, cudaStream_t st);
+// The two launches of a batch's adjoint GEMMs, or loss, on the CUDA cores: the edge of their tiles and about
+// how long they take together; shapes[p] = (k_X, k_Y, d) of pair p
+struct SimtChoice {
+  int tile;   // 32 or 64
+  double us;
+};
+SimtChoice adjoint_simt_choice(const std::vector<int3>& shapes);
+SimtChoice loss_simt_choice(const std::vector<int3>& shapes);
 cudaError_t launch_status_clear(int32_t* status, int n, cudaStream_t st);
 cudaError_t solve_set_smem_limits();
 int64_t chol_factor_floats(int k);   // saved factor size of one row system (padded packed rows)

@@ -372,14 +372,6 @@ cudaError_t adjoint_tc_set_smem() {
   return set_smem_one<1, kLossNt, true>();
 }
 
-// The tensor cores pay from this many flops of a batch per K-block of its longest chain (the two
-// dependent launches together). A K-block costs them about 4.4 us whatever the batch, the FP32
-// tiles run at 13 to 18 TFLOP/s, the tensor cores at 115 once they fill. Launch times in us, FMA
-// tiles against tensor cores: one pair of k = 200, d = 256 23 / 114, 8 of k = 100, d = 384 27 / 68,
-// 64 of k = 100, d = 256 98 / 78, 16 of k = 200 93 / 121, 32 of k = 200 170 / 139, 128 of k = 30
-// 23 / 35; the loss, 4 of k = 200 27 / 82, 32 of k = 200 94 / 85.
-constexpr double kFlopsPerBlock = 88e6;
-
 void adjoint_tc_plan(const std::vector<int3>& shapes, int sms, AdjTcPlan& P) {
   // shapes[p] = (k_X, k_Y, d) of pair p
   auto build = [&](int nt) {
@@ -405,14 +397,23 @@ void adjoint_tc_plan(const std::vector<int3>& shapes, int sms, AdjTcPlan& P) {
   };
   if (P.features == 0) P.features = build(128) >= 2 * sms ? 128 : 64;
   build(P.features);
-  double flops = 0.0;
-  int blocks = 0;
+  // About how long the two launches take: up to 64 columns per CTA the K-blocks of the longest chains
+  // (4 us each, whatever the batch) and a share of every CTA's; wider, all CTAs' K-blocks. The
+  // tensor cores are taken where the FMA tiles would take longer. us, FMA tiles / tensor cores: one pair
+  // of k = 200, d = 256 23 / 113, 128 of k = 30, d = 512 34 / 48, 32, 48, 64 of k = 100, d = 512 71 / 76,
+  // 101 / 82, 121 / 88, 32 and 48 of k = 128 82 / 89, 113 / 94, 16 and 32 of k = 150 74 / 107, 133 / 126, 12
+  // and 16 of k = 300 183 / 190, 238 / 201.
+  int64_t work = 0;
+  int chain = 0;
   for (const int3& q : shapes) {
-    const double k = q.x, ky = q.y, d = q.z;
-    flops += 4.0 * k * k * ky + 2.0 * ky * k * d + 2.0 * k * (ky + k) * d;
-    blocks = std::max(blocks, (std::max(2 * q.y, q.x) + 31) / 32 + (q.x + q.y + 31) / 32);
+    const int k = q.x, ky = q.y, d = q.z, nt = P.features;
+    auto tiles = [&](int m, int n) { return (int64_t)((m + kAdjRows - 1) / kAdjRows) * ((n + nt - 1) / nt); };
+    const int bw = (2 * ky + 31) / 32, bx = (k + ky + 31) / 32, by = (k + 31) / 32;
+    work += tiles(k, k) * bw + tiles(k, d) * bx + tiles(ky, d) * by;
+    chain = std::max(chain, std::max(bw, by) + bx);
   }
-  P.tensor_cores = flops > kFlopsPerBlock * blocks;
+  const double us = P.features <= 64 ? 10.0 + 4.0 * chain + 4e-3 * (double)work : 20.0 + 15e-3 * (double)work;
+  P.tensor_cores = us < adjoint_simt_choice(shapes).us;
   // one stage: twice the CTAs per SM of two stages, which measured faster at every width
   if (P.stages == 0) P.stages = 1;
 }
@@ -452,13 +453,18 @@ void adjoint_tc_loss_plan(const std::vector<int3>& shapes, AdjTcPlan& P) {
   for (const auto& x : e_items) P.items.push_back(x.second);
   for (const auto& x : g_items) P.items.push_back(x.second);
   P.n_first = (int)e_items.size();
-  double flops = 0.0;
-  int blocks = 0;
+  // About how long the two launches take, by all CTAs' K-blocks; taken where the FMA tiles would take
+  // longer; a fifth more where rows of C are not 16-byte aligned (scalar stores). us, FMA tiles / tensor
+  // cores: 32, 64, 96 pairs of k = 200 74 / 84, 131 / 127, 188 / 158, 128 and 256 of k = 100 52 / 57, 88 / 86,
+  // 64 of k = 128 37 / 64, 128 of k = 150 111 / 215, 48 and 64 of k = 250 136 / 160, 157 / 167, 32 of k = 300
+  // 160 / 163.
+  double work = 0.0;
   for (const int3& q : shapes) {
-    flops += 4.0 * q.y * (double)q.y * q.x;
-    blocks = std::max(blocks, (q.x + 31) / 32 + (q.y + 31) / 32);
+    auto tiles = [](int m, int n) { return (int64_t)((m + kAdjRows - 1) / kAdjRows) * ((n + kLossNt - 1) / kLossNt); };
+    work += (double)(tiles(q.y, q.y) * ((q.x + 31) / 32) + tiles(q.y, q.x) * ((q.y + 31) / 32)) *
+            ((q.x | q.y) & 3 ? 1.2 : 1.0);
   }
-  P.tensor_cores = flops > kFlopsPerBlock * blocks;
+  P.tensor_cores = 50.0 + 22.5e-3 * work < loss_simt_choice(shapes).us;
   P.features = kLossNt;
   P.stages = 1;
 }

@@ -7,6 +7,9 @@
 // dA contributions; the training loss; the status clear.
 #include <math.h>
 
+#include <algorithm>
+#include <vector>
+
 #include "fmap_internal.cuh"
 #include "simt_tile.cuh"
 
@@ -21,28 +24,35 @@ __device__ __forceinline__ float mask_entry(const PairDev& pd, const float* evx,
 
 // ---------------------------------------------------------------- adjoint GEMMs
 // Batches that are too small for launch_adjoint_tc, on simt::tile_gemm. Launch times of the two
-// together, 64 x 64 tiles with one chain each -> these: one pair of k = 200, d = 256 0.062 ->
-// 0.023 ms, one of k = 300, d = 512 0.088 -> 0.037, 4 of k = 200, d = 512 0.070 -> 0.045, 8 of
-// k = 100, d = 384 0.043 -> 0.027; the two launches of the loss 0.049 -> 0.023 at k = 300.
-using simt::kT;
+// together, 64 x 64 tiles with one chain and one buffer each -> these: one pair of k = 200, d = 256 62 ->
+// 23 us, one of k = 300, d = 512 88 -> 38, 4 of k = 200, d = 512 72 -> 48, 8 of k = 100, d = 512 44 -> 31,
+// 32 of k = 100 80 -> 71; the two launches of the loss 48 -> 21 at k = 300, 32 pairs of k = 200 97 -> 74.
 using simt::Operand;
+using simt::out_col;
+using simt::out_row;
+using simt::Tile;
 
 // W = Gamma^T C + C^T Gamma (k_X x k_X; Gamma and C are k_Y x k_X).
+template <int kT>
 __global__ void __launch_bounds__(simt::kThreads) adjoint_w_kernel(BatchDev b, const float* c_flat, float* ws) {
-  __shared__ __align__(16) simt::Smem sm;
+  __shared__ __align__(16) typename Tile<kT>::Smem sm;
   const PairDev pd = b.pairs[blockIdx.y];
   const int k = pd.k, ky = b.shapes[pd.y].k;   // Gamma, C: ky x k
   const int nt = (k + kT - 1) / kT;
   if ((int)blockIdx.x >= nt * nt) return;
   const int a0 = (blockIdx.x / nt) * kT, b0 = (blockIdx.x % nt) * kT;
   const Operand gam{ws + pd.gam_off, k, k, ky}, c{c_flat + pd.c_off, k, k, ky};
-  const float4 v = simt::tile_gemm<false, false>(sm, gam, c, c, gam, 1.f, a0, b0);
-  const int i = a0 + (threadIdx.x >> 3), j = b0 + 4 * (threadIdx.x & 7);
-  float* w = ws + pd.w_off + (int64_t)i * k + j;
-  const float o[4] = {v.x, v.y, v.z, v.w};
+  float v[Tile<kT>::kRows][4];
+  simt::tile_gemm<kT, simt::kAcross, simt::kAcross>(sm, gam, c, c, gam, 1.f, a0, b0, v);
+  const int j = b0 + out_col<kT>();
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (i < k && j + q < k) w[q] = o[q];
+  for (int u = 0; u < Tile<kT>::kRows; ++u) {
+    const int i = a0 + out_row<kT>(u);
+    float* w = ws + pd.w_off + (int64_t)i * k + j;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i < k && j + q < k) w[q] = v[u][q];
+  }
 }
 
 // The mask gradient dD = -lambda_i Gamma o C (when d_mask is given; lambda_i = lambda
@@ -96,8 +106,9 @@ __global__ void __launch_bounds__(256) adjoint_dlambda_kernel(BatchDev b, const 
 // Per-pair contributions (Gamma is k_Y x k_X, W k_X x k_X and symmetric):
 //   which 0: dA_x = Gamma^T A_y - W A_x   (k_X x d, into sx_off)
 //   which 1: dA_y = Gamma A_x             (k_Y x d, into sy_off)
+template <int kT>
 __global__ void __launch_bounds__(simt::kThreads) adjoint_da_kernel(BatchDev b, const float* a_flat, float* ws) {
-  __shared__ __align__(16) simt::Smem sm;
+  __shared__ __align__(16) typename Tile<kT>::Smem sm;
   const PairDev pd = b.pairs[blockIdx.y];
   const int k = pd.k, ky = b.shapes[pd.y].k, d = pd.d;
   const int which = blockIdx.z;
@@ -107,15 +118,20 @@ __global__ void __launch_bounds__(simt::kThreads) adjoint_da_kernel(BatchDev b, 
   const int a0 = (blockIdx.x / ntf) * kT, f0 = (blockIdx.x % ntf) * kT;
   const float* gam = ws + pd.gam_off;
   const Operand ax{a_flat + b.shapes[pd.x].a_off, d, d, k}, ay{a_flat + b.shapes[pd.y].a_off, d, d, ky};
-  float4 v;
+  float v[Tile<kT>::kRows][4];
   if (which == 0)
-    v = simt::tile_gemm<false, false>(sm, Operand{gam, k, k, ky}, ay, Operand{ws + pd.w_off, k, k, k}, ax, -1.f, a0, f0);
+    simt::tile_gemm<kT, simt::kAcross, simt::kAcross>(sm, Operand{gam, k, k, ky}, ay, Operand{ws + pd.w_off, k, k, k}, ax, -1.f, a0, f0, v);
   else
-    v = simt::tile_gemm<true, false>(sm, Operand{gam, k, ky, k}, ax, Operand{nullptr, 0, 0, 0}, Operand{nullptr, 0, 0, 0},
-                                     1.f, a0, f0);
-  const int i = a0 + (threadIdx.x >> 3), f = f0 + 4 * (threadIdx.x & 7);
-  // d is a multiple of 16 and the contributions are 256-byte aligned
-  if (i < rows && f < d) *reinterpret_cast<float4*>(ws + (which == 0 ? pd.sx_off : pd.sy_off) + (int64_t)i * d + f) = v;
+    simt::tile_gemm<kT, simt::kQuads, simt::kAcross>(sm, Operand{gam, k, ky, k}, ax, Operand{nullptr, 0, 0, 0}, Operand{nullptr, 0, 0, 0},
+                                     1.f, a0, f0, v);
+  const int f = f0 + out_col<kT>();
+  float* out = ws + (which == 0 ? pd.sx_off : pd.sy_off) + f;
+#pragma unroll
+  for (int u = 0; u < Tile<kT>::kRows; ++u) {
+    const int i = a0 + out_row<kT>(u);
+    // d is a multiple of 16 and the contributions are 256-byte aligned
+    if (i < rows && f < d) *reinterpret_cast<float4*>(out + (int64_t)i * d) = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
+  }
 }
 
 // dA_s = sum of the shape's contributions, in pair order. Each thread sums four
@@ -145,13 +161,14 @@ __global__ void gather_da_kernel(BatchDev b, float* d_a, const float* ws) {
 }
 
 // Training loss ||C C^T - I||^2 + ||C - C_gt||^2 and dL/dC = 4 (C C^T - I) C + 2 (C - C_gt),
-// as two tiled passes over (32 x 32 output tile, pair):
+// as two tiled passes over (output tile, pair):
 //   pass 1: E = C C^T - I (into the workspace) and per-tile partial sums of the loss;
 //   pass 2: dC = 4 E C + 2 (C - C_gt); tile 0 of each pair adds the partials in a fixed order.
 
+template <int kT>
 __global__ void __launch_bounds__(simt::kThreads) loss_e_kernel(BatchDev b, const float* c_flat, const float* gt_flat,
                                                                 float* ws, float* partial) {
-  __shared__ __align__(16) simt::Smem sm;
+  __shared__ __align__(16) typename Tile<kT>::Smem sm;
   __shared__ float red[simt::kThreads];
   const int p = blockIdx.y;
   const PairDev pd = b.pairs[p];
@@ -167,21 +184,24 @@ __global__ void __launch_bounds__(simt::kThreads) loss_e_kernel(BatchDev b, cons
   const int tid = threadIdx.x;
   const Operand none{nullptr, 0, 0, 0};
   const Operand cr{c, k, ky, b0 < ky ? k : 0};   // no products in the tiles past E's columns
-  const float4 v4 = simt::tile_gemm<true, true>(sm, cr, cr, none, none, 1.f, a0, b0);
-  const float v[4] = {v4.x, v4.y, v4.z, v4.w};
-  const int a = a0 + (tid >> 3);
+  float v[Tile<kT>::kRows][4];
+  simt::tile_gemm<kT, simt::kLanes, simt::kLanes>(sm, cr, cr, none, none, 1.f, a0, b0, v);
   float part = 0.f;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int bb = b0 + 4 * (tid & 7) + j;
-    if (a < ky && bb < k) {
-      const float r = c[(int64_t)a * k + bb] - gt[(int64_t)a * k + bb];
-      part = fmaf(r, r, part);
-    }
-    if (a < ky && bb < ky) {
-      const float x = v[j] - (a == bb ? 1.f : 0.f);
-      e[(int64_t)a * ky + bb] = x;
-      part = fmaf(x, x, part);
+  for (int u = 0; u < Tile<kT>::kRows; ++u) {
+    const int a = a0 + out_row<kT>(u);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int bb = b0 + out_col<kT>() + j;
+      if (a < ky && bb < k) {
+        const float r = c[(int64_t)a * k + bb] - gt[(int64_t)a * k + bb];
+        part = fmaf(r, r, part);
+      }
+      if (a < ky && bb < ky) {
+        const float x = v[u][j] - (a == bb ? 1.f : 0.f);
+        e[(int64_t)a * ky + bb] = x;
+        part = fmaf(x, x, part);
+      }
     }
   }
   red[tid] = part;
@@ -193,10 +213,11 @@ __global__ void __launch_bounds__(simt::kThreads) loss_e_kernel(BatchDev b, cons
   if (tid == 0) partial[(int64_t)p * kMaxLossTiles + blockIdx.x] = red[0];
 }
 
+template <int kT>
 __global__ void __launch_bounds__(simt::kThreads) loss_grad_kernel(BatchDev b, const float* c_flat, const float* gt_flat,
                                                                    float* loss, float* d_c, const float* ws,
                                                                    const float* partial) {
-  __shared__ __align__(16) simt::Smem sm;
+  __shared__ __align__(16) typename Tile<kT>::Smem sm;
   const int p = blockIdx.y;
   const PairDev pd = b.pairs[p];
   const int k = pd.k, ky = b.shapes[pd.y].k;
@@ -217,16 +238,18 @@ __global__ void __launch_bounds__(simt::kThreads) loss_grad_kernel(BatchDev b, c
   const float* c = c_flat + pd.c_off;
   const float* gt = gt_flat + pd.c_off;
   const Operand none{nullptr, 0, 0, 0};
-  const float4 v4 = simt::tile_gemm<true, false>(sm, Operand{ws + pd.e_off, ky, ky, ky}, Operand{c, k, k, ky}, none,
-                                                 none, 1.f, a0, b0);
-  const float v[4] = {v4.x, v4.y, v4.z, v4.w};
-  const int a = a0 + (threadIdx.x >> 3);
+  float v[Tile<kT>::kRows][4];
+  simt::tile_gemm<kT, simt::kLanes, simt::kAcross>(sm, Operand{ws + pd.e_off, ky, ky, ky}, Operand{c, k, k, ky}, none, none, 1.f, a0, b0, v);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int bb = b0 + 4 * (threadIdx.x & 7) + j;
-    if (a >= ky || bb >= k) continue;
-    const int64_t idx = (int64_t)a * k + bb;
-    d_c[pd.c_off + idx] = 4.f * v[j] + 2.f * (c[idx] - gt[idx]);
+  for (int u = 0; u < Tile<kT>::kRows; ++u) {
+    const int a = a0 + out_row<kT>(u);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int bb = b0 + out_col<kT>() + j;
+      if (a >= ky || bb >= k) continue;
+      const int64_t idx = (int64_t)a * k + bb;
+      d_c[pd.c_off + idx] = 4.f * v[u][j] + 2.f * (c[idx] - gt[idx]);
+    }
   }
 }
 
@@ -237,22 +260,73 @@ __global__ void status_clear_kernel(int32_t* status, int n) {
 
 }  // namespace
 
+namespace {
+
+// Tiles of edge t of an m x n output.
+int64_t tiles_of(int m, int n, int t) { return (int64_t)((m + t - 1) / t) * ((n + t - 1) / t); }
+int slabs_of(int len) { return (len + simt::kS - 1) / simt::kS; }
+
+}  // namespace
+
+// Which tile, for both: 64 x 64 once the 32 x 32 tiles are more than the SMs hold at a time (six
+// blocks each) and at least 3.2 times as many (an edge that 64 pads to much more than 32 does stays
+// with 32). Times in us, 32 / 64: the loss of 32, 48, 64, 128 pairs of k = 100 26 / 26, 31 / 34, 38 / 35,
+// 62 / 52, of 16 and 32 of k = 250 58 / 56, 103 / 91, of 64 of k = 90 (ratio 2.25) 26 / 32; the adjoint
+// (d = 512) of 12, 24, 48 of k = 100 41 / 43, 65 / 60, 121 / 101, of 16 and 32 of k = 128 52 / 56,
+// 88 / 82, of 32 and 64 of k = 64 32 / 32, 53 / 47, of 32 of k = 77 (ratio 3) 48 / 51, of 32 and 64 of k = 150
+// (ratio 3.3) 133 / 135, 249 / 242. For the adjoint the line is at fifteen tiles of dA per SM (its reductions
+// are longer) and a ratio of 3.5.
+SimtChoice loss_simt_choice(const std::vector<int3>& shapes) {
+  int64_t n32 = 0, n64 = 0, w32 = 0, w64 = 0;   // tiles of E; tiles times slabs of both launches
+  for (const int3& q : shapes) {
+    const int k = q.x, ky = q.y;
+    n32 += tiles_of(ky, std::max(k, ky), 32);
+    n64 += tiles_of(ky, std::max(k, ky), 64);
+    w32 += tiles_of(ky, ky, 32) * slabs_of(k) + tiles_of(ky, k, 32) * slabs_of(ky);
+    w64 += tiles_of(ky, ky, 64) * slabs_of(k) + tiles_of(ky, k, 64) * slabs_of(ky);
+  }
+  if (n32 > 6 * 152 && 10 * n32 > 32 * n64) return {64, 10.0 + 4.75e-3 * (double)w64};
+  return {32, 10.0 + 1.55e-3 * (double)w32};
+}
+
+SimtChoice adjoint_simt_choice(const std::vector<int3>& shapes) {
+  int64_t n32 = 0, n64 = 0, w32 = 0, w64 = 0;   // tiles of dA; tiles times slabs of both launches
+  for (const int3& q : shapes) {
+    const int k = q.x, ky = q.y, d = q.z;
+    n32 += tiles_of(k, d, 32) + tiles_of(ky, d, 32);
+    n64 += tiles_of(k, d, 64) + tiles_of(ky, d, 64);
+    const int sw = 2 * slabs_of(ky), sx = slabs_of(ky) + slabs_of(k), sy = slabs_of(k);
+    w32 += tiles_of(k, k, 32) * sw + tiles_of(k, d, 32) * sx + tiles_of(ky, d, 32) * sy;
+    w64 += tiles_of(k, k, 64) * sw + tiles_of(k, d, 64) * sx + tiles_of(ky, d, 64) * sy;
+  }
+  if (n32 > 15 * 152 && 10 * n32 > 35 * n64) return {64, 15.0 + 4.7e-3 * (double)w64};
+  return {32, 10.0 + 1.5e-3 * (double)w32};
+}
+
 cudaError_t launch_adjoint_gemms(const BatchDev& b, int max_k, int max_d, const float* a, const float* c,
-                                 float* d_mask, float* d_lambda, bool row_grads, float* ws, bool simt,
+                                 float* d_mask, float* d_lambda, bool row_grads, float* ws, int simt_tile,
                                  cudaStream_t st) {
   if (b.n_pairs <= 0) return cudaSuccess;
-  const int ntk = (max_k + kT - 1) / kT, ntd = (max_d + kT - 1) / kT;
+  auto tiles = [&](int n) { return (n + simt_tile - 1) / simt_tile; };
   cudaError_t e;
-  if (simt) {
-    adjoint_w_kernel<<<dim3(ntk * ntk, b.n_pairs), simt::kThreads, 0, st>>>(b, c, ws);
+  if (simt_tile) {
+    const dim3 grid(tiles(max_k) * tiles(max_k), b.n_pairs);
+    if (simt_tile == 64)
+      adjoint_w_kernel<64><<<grid, simt::kThreads, 0, st>>>(b, c, ws);
+    else
+      adjoint_w_kernel<32><<<grid, simt::kThreads, 0, st>>>(b, c, ws);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (d_lambda || d_mask || row_grads) {
     adjoint_dlambda_kernel<<<b.n_pairs, 256, 0, st>>>(b, c, d_mask, d_lambda, ws);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if (!simt) return cudaSuccess;
-  adjoint_da_kernel<<<dim3(ntk * ntd, b.n_pairs, 2), simt::kThreads, 0, st>>>(b, a, ws);
+  if (!simt_tile) return cudaSuccess;
+  const dim3 grid(tiles(max_k) * tiles(max_d), b.n_pairs, 2);
+  if (simt_tile == 64)
+    adjoint_da_kernel<64><<<grid, simt::kThreads, 0, st>>>(b, a, ws);
+  else
+    adjoint_da_kernel<32><<<grid, simt::kThreads, 0, st>>>(b, a, ws);
   return cudaGetLastError();
 }
 
@@ -263,13 +337,20 @@ cudaError_t launch_gather_da(const BatchDev& b, int max_kd, float* d_a, const fl
 }
 
 cudaError_t launch_loss_orth(const BatchDev& b, int max_k, const float* c, const float* c_gt, float* loss,
-                             float* d_c, float* ws, float* partial, cudaStream_t st) {
+                             float* d_c, float* ws, float* partial, int simt_tile, cudaStream_t st) {
   if (b.n_pairs <= 0) return cudaSuccess;
-  const int nt = (max_k + kT - 1) / kT;
-  loss_e_kernel<<<dim3(nt * nt, b.n_pairs), simt::kThreads, 0, st>>>(b, c, c_gt, ws, partial);
+  const int nt = (max_k + simt_tile - 1) / simt_tile;
+  const dim3 grid(nt * nt, b.n_pairs);
+  if (simt_tile == 64)
+    loss_e_kernel<64><<<grid, simt::kThreads, 0, st>>>(b, c, c_gt, ws, partial);
+  else
+    loss_e_kernel<32><<<grid, simt::kThreads, 0, st>>>(b, c, c_gt, ws, partial);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  loss_grad_kernel<<<dim3(nt * nt, b.n_pairs), simt::kThreads, 0, st>>>(b, c, c_gt, loss, d_c, ws, partial);
+  if (simt_tile == 64)
+    loss_grad_kernel<64><<<grid, simt::kThreads, 0, st>>>(b, c, c_gt, loss, d_c, ws, partial);
+  else
+    loss_grad_kernel<32><<<grid, simt::kThreads, 0, st>>>(b, c, c_gt, loss, d_c, ws, partial);
   return cudaGetLastError();
 }
 

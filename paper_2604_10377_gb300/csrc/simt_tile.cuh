@@ -1,9 +1,10 @@
-// 32 x 32 output tiles of small FP32 GEMMs on the CUDA cores, 256 threads, 4 x 4 outputs per
-// thread: four groups of 64 threads take every fourth slab of 16 reduction indices, and their
-// sums are added in order at the end. The batches these serve do not fill the SMs, so the chain
-// of a tile (a global load, a slab through shared memory, 16 steps of FMAs, a barrier) bounds a
-// launch; the split makes it a quarter as long as one chain per tile, and a tile a quarter of
-// 64 x 64 spreads it over four times the SMs.
+// Output tiles of FP32 GEMMs on the CUDA cores, 256 threads, 4 x 4 outputs per thread, slabs of 16
+// reduction indices through shared memory:
+//   32 x 32  four groups of 64 threads take every fourth slab, and their sums are added in order at the
+//            end. For batches that do not fill the SMs, where the chain of a tile (a global load, a
+//            slab through shared memory, 16 steps of FMAs, a barrier) bounds a launch: it is a quarter
+//            as long, and spread over four times the SMs.
+//   64 x 64  one group of 256 threads takes every slab: half the loads per product.
 #pragma once
 
 #include <stdint.h>
@@ -13,92 +14,146 @@
 namespace fmap {
 namespace simt {
 
-constexpr int kT = 32;         // tile edge
 constexpr int kS = 16;         // reduction indices per slab
-constexpr int kGroups = 4;
-constexpr int kThreads = 64 * kGroups;
-constexpr int kLd = kT + 4;
+constexpr int kThreads = 256;
 
-union Smem {
-  float slab[kGroups][2][2][kS][kLd];   // group, buffer, operand, reduction index, row
-  float part[kGroups][kT][kT];          // group, row, column
+template <int kTile>
+struct Tile {
+  static_assert(kTile == 32 || kTile == 64, "tile edge");
+  static constexpr int kGroup = (kTile / 4) * (kTile / 4);     // threads of a group
+  static constexpr int kGroups = kThreads / kGroup;
+  static constexpr int kPer = kTile * kS / 4 / kGroup;         // quads of an operand's slab per thread
+  static constexpr int kLd = kTile + 4;
+  static constexpr int kRows = kTile * kTile / 4 / kThreads;   // quads of the tile per thread at the end
+  union Smem {
+    float slab[kGroups][2][2][kS][kLd];                        // group, buffer, operand, reduction index, row
+    float part[kGroups > 1 ? kGroups : 1][kGroups > 1 ? kTile : 1][kTile];   // group, row, column
+  };
 };
 
+// Row and first column, within the tile, of quad i of this thread's results.
+template <int kTile>
+__device__ __forceinline__ int out_row(int i) {
+  return kTile == 32 ? threadIdx.x >> 3 : 4 * (threadIdx.x >> 4) + i;
+}
+template <int kTile>
+__device__ __forceinline__ int out_col() {
+  return 4 * (threadIdx.x & (kTile / 4 - 1));
+}
+
 // An operand: element (r, m) of `rows` x `len` (r an output row or column, m the reduction index)
-// at p[r ld + m] (kContig) or p[m ld + r].
+// at p[m ld + r] (kAcross) or p[r ld + m]. The latter is read in quads of a row, which take few addresses (the
+// adjoint's dA_y at d = 512: 4 pairs of k = 100 23 us against 25, 128 of k = 64 71 against 75), or by 16
+// lanes along a row, whose loads touch a quarter of the lines (the loss, where both operands are so: 128
+// pairs of k = 100 72 -> 62 us in tiles of 32, 58 -> 52 in tiles of 64).
+enum Layout { kAcross, kQuads, kLanes };
 struct Operand {
   const float* p;
   int64_t ld;
   int rows, len;
 };
 
+template <int kTile>
 __device__ __forceinline__ void group_sync(int g) {   // constant ids: a variable one reserves all sixteen
+  if (Tile<kTile>::kGroups == 1) {
+    __syncthreads();
+  } else {
 #pragma unroll
-  for (int u = 0; u < kGroups; ++u)
-    if (g == u) tc::named_barrier_sync(1 + u, 64);
+    for (int u = 0; u < Tile<kTile>::kGroups; ++u)
+      if (g == u) tc::named_barrier_sync(1 + u, Tile<kTile>::kGroup);
+  }
 }
 
-// Slab values of thread t (0 .. 63): two quads. kContig: indices m0 + 4 (t & 3) .. + 3 of rows
-// r0 + t / 4 and + 16; else rows r0 + 4 (t & 7) .. + 3 of indices m0 + t / 8 and + 8.
-template <bool kContig>
-__device__ __forceinline__ void fetch_slab(const Operand& o, int r0, int m0, int t, float (&v)[2][4]) {
+// Row and reduction index, within the slab, of value j of quad u of thread t of a group.
+template <int kTile, Layout kL>
+__device__ __forceinline__ void slab_at(int t, int u, int j, int& r, int& m) {
+  constexpr int kG = Tile<kTile>::kGroup, kQ = kTile / 4;
+  if (kL == kAcross) {
+    r = 4 * (t & (kQ - 1)) + j;
+    m = t / kQ + kG / kQ * u;
+  } else if (kL == kQuads) {
+    r = (t >> 2) + kG / 4 * u;
+    m = 4 * (t & 3) + j;
+  } else {
+    r = (t >> 4) + kG / 16 * (4 * u + j);
+    m = t & 15;
+  }
+}
+
+template <int kTile, Layout kL>
+__device__ __forceinline__ void fetch_slab(const Operand& o, int r0, int m0, int t, float (&v)[Tile<kTile>::kPer][4]) {
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int r = kContig ? r0 + (t >> 2) + 16 * u : r0 + 4 * (t & 7);
-    const int m = kContig ? m0 + 4 * (t & 3) : m0 + (t >> 3) + 8 * u;
-    const float* q = kContig ? o.p + (int64_t)r * o.ld + m : o.p + (int64_t)m * o.ld + r;
+  for (int u = 0; u < Tile<kTile>::kPer; ++u) {
+    int r, m;
+    slab_at<kTile, kL>(t, u, 0, r, m);
+    r += r0;
+    m += m0;
+    const float* q = kL == kAcross ? o.p + (int64_t)m * o.ld + r : o.p + (int64_t)r * o.ld + m;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const bool ok = kContig ? (r < o.rows && m + j < o.len) : (m < o.len && r + j < o.rows);
-      v[u][j] = ok ? __ldg(q + j) : 0.f;
+      if (kL == kLanes) {
+        slab_at<kTile, kL>(t, u, j, r, m);
+        r += r0;
+        m += m0;
+        v[u][j] = r < o.rows && m < o.len ? __ldg(o.p + (int64_t)r * o.ld + m) : 0.f;
+      } else {
+        v[u][j] = (kL == kAcross ? m < o.len && r + j < o.rows : r < o.rows && m + j < o.len) ? __ldg(q + j) : 0.f;
+      }
     }
   }
 }
 
-template <bool kContig>
-__device__ __forceinline__ void store_slab(float (*s)[kLd], int t, const float (&v)[2][4]) {
+template <int kTile, Layout kL>
+__device__ __forceinline__ void store_slab(float (*s)[Tile<kTile>::kLd], int t, const float (&v)[Tile<kTile>::kPer][4]) {
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    if (kContig) {
-      const int r = (t >> 2) + 16 * u, m = 4 * (t & 3);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s[m + j][r] = v[u][j];
+  for (int u = 0; u < Tile<kTile>::kPer; ++u) {
+    int r, m;
+    if (kL == kAcross) {
+      slab_at<kTile, kL>(t, u, 0, r, m);
+      *reinterpret_cast<float4*>(&s[m][r]) = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
     } else {
-      *reinterpret_cast<float4*>(&s[(t >> 3) + 8 * u][4 * (t & 7)]) = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        slab_at<kTile, kL>(t, u, j, r, m);
+        s[m][r] = v[u][j];
+      }
     }
   }
 }
 
 // sum_m X1(i0 + i, m) Y1(j0 + j, m) + sign2 sum_m X2(i0 + i, m) Y2(j0 + j, m) for one tile (the
-// second term absent when X2.len is 0). Thread t returns columns 4 (t & 7) .. + 3 of row t / 8.
-template <bool kXContig, bool kYContig>
-__device__ __forceinline__ float4 tile_gemm(Smem& sm, const Operand& x1, const Operand& y1, const Operand& x2,
-                                            const Operand& y2, float sign2, int i0, int j0) {
-  const int tid = threadIdx.x, g = tid >> 6, t = tid & 63, tx = t & 7, ty = t >> 3;
+// second term absent when X2.len is 0): out[q] is the quad at (out_row(q), out_col()).
+template <int kTile, Layout kX, Layout kY>
+__device__ __forceinline__ void tile_gemm(typename Tile<kTile>::Smem& sm, const Operand& x1, const Operand& y1,
+                                          const Operand& x2, const Operand& y2, float sign2, int i0, int j0,
+                                          float (&out)[Tile<kTile>::kRows][4]) {
+  using T = Tile<kTile>;
+  const int tid = threadIdx.x, g = tid / T::kGroup, t = tid & (T::kGroup - 1);
+  const int tx = t & (kTile / 4 - 1), ty = t / (kTile / 4);
   float acc[4][4] = {};
   const int n1 = (x1.len + kS - 1) / kS, n = n1 + (x2.len + kS - 1) / kS;
-  float rx[2][4], ry[2][4];
+  float rx[T::kPer][4], ry[T::kPer][4];
   auto fetch = [&](int sl) {
     const bool second = sl >= n1;
     const int m0 = (second ? sl - n1 : sl) * kS;
-    fetch_slab<kXContig>(second ? x2 : x1, i0, m0, t, rx);
-    fetch_slab<kYContig>(second ? y2 : y1, j0, m0, t, ry);
+    fetch_slab<kTile, kX>(second ? x2 : x1, i0, m0, t, rx);
+    fetch_slab<kTile, kY>(second ? y2 : y1, j0, m0, t, ry);
   };
   if (g < n) fetch(g);
   int buf = 0;
-  for (int sl = g; sl < n; sl += kGroups, buf ^= 1) {
-    float(*sx)[kLd] = sm.slab[g][buf][0];
-    float(*sy)[kLd] = sm.slab[g][buf][1];
+  for (int sl = g; sl < n; sl += T::kGroups, buf ^= 1) {
+    float(*sx)[T::kLd] = sm.slab[g][buf][0];
+    float(*sy)[T::kLd] = sm.slab[g][buf][1];
     if (sl >= n1) {
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
+      for (int u = 0; u < T::kPer; ++u)
 #pragma unroll
         for (int j = 0; j < 4; ++j) rx[u][j] *= sign2;
     }
-    store_slab<kXContig>(sx, t, rx);
-    store_slab<kYContig>(sy, t, ry);
-    group_sync(g);   // (the other buffer's readers passed it one slab ago)
-    if (sl + kGroups < n) fetch(sl + kGroups);
+    store_slab<kTile, kX>(sx, t, rx);
+    store_slab<kTile, kY>(sy, t, ry);
+    group_sync<kTile>(g);   // (the other buffer's readers passed it one slab ago)
+    if (sl + T::kGroups < n) fetch(sl + T::kGroups);
 #pragma unroll
     for (int c = 0; c < kS; ++c) {
       const float4 xa = *reinterpret_cast<const float4*>(&sx[c][ty * 4]);
@@ -110,18 +165,25 @@ __device__ __forceinline__ float4 tile_gemm(Smem& sm, const Operand& x1, const O
         for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(xv[a], yv[b], acc[a][b]);
     }
   }
-  __syncthreads();   // every group has read its slabs
+  if constexpr (T::kGroups == 1) {
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
-    *reinterpret_cast<float4*>(&sm.part[g][4 * ty + a][4 * tx]) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
-  __syncthreads();
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-  for (int u = 0; u < kGroups; ++u) {
-    const float4 w = *reinterpret_cast<const float4*>(&sm.part[u][tid >> 3][4 * (tid & 7)]);
-    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+      for (int b = 0; b < 4; ++b) out[a][b] = acc[a][b];
+  } else {
+    __syncthreads();   // every group has read its slabs
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+      *reinterpret_cast<float4*>(&sm.part[g][4 * ty + a][4 * tx]) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+    __syncthreads();
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < T::kGroups; ++u) {
+      const float4 w = *reinterpret_cast<const float4*>(&sm.part[u][out_row<kTile>(0)][out_col<kTile>()]);
+      v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+    }
+    out[0][0] = v.x; out[0][1] = v.y; out[0][2] = v.z; out[0][3] = v.w;
   }
-  return v;
 }
 
 }  // namespace simt
