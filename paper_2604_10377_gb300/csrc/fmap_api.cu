@@ -92,7 +92,7 @@ struct Plan {
   std::vector<TcLaunch> tc_launches;
   std::vector<TcRedGroup> tc_groups;
   std::vector<int64_t> tc_parts;       // offsets of the partials, group after group
-  int64_t tc_max_group_elems = 0;
+  int64_t tc_max_group_blocks = 0;     // blocks of the reduction for its largest group
   // tensor-core backward projection
   std::vector<TcBwdItem> bw_items;
   std::vector<int32_t> bw_cta_first;   // bwd_ctas + 1 (FP32) or bwd_ctas / 2 + 1 (BF16) boundaries
@@ -308,7 +308,8 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
         }
         rg.part_end = (int32_t)P.tc_parts.size();
         P.tc_groups.push_back(rg);
-        P.tc_max_group_elems = std::max<int64_t>(P.tc_max_group_elems, (int64_t)u.nk * rg.dspan);
+        const int64_t red_per = 4 * 256 / tc_red_subs(rg.part_end - rg.part_beg);
+        P.tc_max_group_blocks = std::max<int64_t>(P.tc_max_group_blocks, ((int64_t)u.nk * rg.dspan + red_per - 1) / red_per);
       }
       for (int c = cta + 1; c <= nctas; ++c) first[c] = (int32_t)P.tc_items.size();
       L.f_stage = fmax * (uint32_t)stage_v;
@@ -978,7 +979,7 @@ int32_t fmap_project(fmap_batch* b, float* a_out, void* ws, size_t ws_bytes, voi
   {
     TimedScope ts(b, FMAP_KIND_PROJECT_REDUCE, st);
     e = launch_project_tc_reduce(b->dev.shapes, b->d_tc_parts, b->d_tc_groups, (int)P.tc_groups.size(),
-                                 P.tc_max_group_elems, a_out, w, st);
+                                 P.tc_max_group_blocks, a_out, w, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "project_reduce");
   return FMAP_OK;

@@ -189,8 +189,10 @@ cudaError_t project_tc32_set_smem(int bytes);
 cudaError_t launch_project_tc32(const TcProjParams& p, int grid, int smem_bytes, cudaStream_t st);
 cudaError_t launch_project_tc(const TcProjParams& p, int grid, int smem_bytes, cudaStream_t st);
 cudaError_t launch_project_tc_reduce(const ShapeDev* shapes, const int64_t* parts, const TcRedGroup* groups,
-                                     int n_groups, int64_t max_elems, float* a_out, const float* ws,
-                                     cudaStream_t st);
+                                     int n_groups, int64_t max_blocks, float* a_out, const float* ws, cudaStream_t st);
+// Thread groups that share the partials of an element of A, by their number; a block of 256 threads
+// takes 256 / tc_red_subs elements of four floats.
+__host__ __device__ constexpr int tc_red_subs(int parts) { return parts < 16 ? 1 : 4; }
 
 // ---- launchers (each enqueues on `st`; return cudaError_t of the launch) ----
 // with_r = false computes G only (the adjoint solves never read R)

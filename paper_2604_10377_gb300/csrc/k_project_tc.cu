@@ -319,13 +319,14 @@ __global__ void __launch_bounds__(256) project_tc_reduce_kernel(const ShapeDev* 
                                                                 const TcRedGroup* groups, float* a_out, const float* ws) {
   __shared__ float4 red[3][64];
   const TcRedGroup g = groups[blockIdx.y];
-  const ShapeDev s = shapes[g.shape];
   // four consecutive features per thread (dspan, f0, d are multiples of 16 and the
   // partials are 256-byte aligned; float4 stores when the output buffer is 16-byte aligned)
   const int q4 = g.dspan >> 2, total = g.nk * q4;
+  const int subs = tc_red_subs(g.part_end - g.part_beg), per = 256 / subs;      // thread groups, elements of each
+  if ((int)blockIdx.x * per >= total) return;
+  const ShapeDev s = shapes[g.shape];
   const bool vec = (reinterpret_cast<uintptr_t>(a_out) & 15) == 0;
   float* out = a_out + s.a_off + (int64_t)g.n0 * s.d + g.f0;
-  const int subs = g.part_end - g.part_beg < 16 ? 1 : 4, per = 256 / subs;      // thread groups, elements of each
   const int sub = threadIdx.x / per, lane = threadIdx.x - sub * per;
   for (int e0 = blockIdx.x * per; e0 < total; e0 += gridDim.x * per) {
     const int e = e0 + lane;
@@ -382,10 +383,9 @@ cudaError_t launch_project_tc(const TcProjParams& p, int grid, int smem_bytes, c
 }
 
 cudaError_t launch_project_tc_reduce(const ShapeDev* shapes, const int64_t* parts, const TcRedGroup* groups,
-                                     int n_groups, int64_t max_elems, float* a_out, const float* ws,
-                                     cudaStream_t st) {
+                                     int n_groups, int64_t max_blocks, float* a_out, const float* ws, cudaStream_t st) {
   if (n_groups <= 0) return cudaSuccess;
-  dim3 grid((unsigned)std::min<int64_t>((max_elems / 4 + 63) / 64, 4096), (unsigned)n_groups);
+  dim3 grid((unsigned)std::min<int64_t>(max_blocks, 4096), (unsigned)n_groups);
   project_tc_reduce_kernel<<<grid, 256, 0, st>>>(shapes, parts, groups, a_out, ws);
   return cudaGetLastError();
 }
