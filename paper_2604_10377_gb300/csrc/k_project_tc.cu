@@ -20,8 +20,9 @@
 // come next, each of which reads the F tile and takes its time to issue. 64 shapes of n = 50000,
 // d = 256 at k = 30 / 50 / 100 / 200: 433 / 454 / 500 / 789 us with separate MMAs for hi and lo,
 // descriptors built between them, one lane issuing all copies and two stages of 64 vertices at
-// k = 200; 380 / 405 / 470 / 771 with one MMA; 335 / 367 / 445 / 658 with descriptors ahead of
-// the waits, a lane per copy and stages of 32 where three of 64 do not fit.
+// k = 200; 380 / 405 / 470 / 771 with one MMA; 335 / 364 / 442 / 642 with descriptors ahead of
+// the waits, a lane per copy and stages of 32 where three of 64 do not fit. (With one feature group,
+// d <= 128, the conversion of Phi bounds it from k = 176 on: 32 shapes of k = 200, d = 128 277 us.)
 // At the end of a segment warps 2-9 read the accumulators back (tcgen05.ld) and
 // write the segment's partial A; a second kernel adds the partials of each shape
 // in a fixed order. F is exact in BF16, so A carries only the ~2^-17 error of
@@ -50,13 +51,13 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint3
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// The MMAs of one segment. kV: vertices per stage; kFg: feature groups (0: item.fg); kMerged: tc_merged. One
-// lane issues them and the time per MMA counts at small k, so the descriptors are computed ahead of the waits.
+// The MMAs of one segment. kV: vertices per stage; kFg: feature groups (0: item.fg); kMerged: tc_merged. The
+// time per MMA counts at small k, so the descriptors are computed ahead of the waits. (One thread alone waits
+// and issues: with its warp waiting beside it 16 shapes of n = 50000, k = 200, d = 256 take 177 us, not 171.)
 template <int kV, int kFg, bool kMerged>
-__device__ __forceinline__ bool issue(const TcProjParams& P, const TcItem& item, int nst, uint32_t tmem_base, uint8_t* sF,
+__device__ __forceinline__ bool issue_by_one_thread(const TcProjParams& P, const TcItem& item, int nst, uint32_t tmem_base, uint8_t* sF,
                                       uint8_t* sP, uint64_t* full_f, uint64_t* full_p, uint64_t* empty, uint32_t& stage,
                                       uint32_t& phase, volatile int* abort) {
-  const bool lead = (threadIdx.x & 31) == 0;
   const int fg = kFg ? kFg : item.fg;
   const uint32_t npad = (uint32_t)item.npad;
   const uint32_t cols = npad * (kMerged ? 2u : 1u);      // accumulator columns per feature group
@@ -65,7 +66,7 @@ __device__ __forceinline__ bool issue(const TcProjParams& P, const TcItem& item,
   for (int st = 0; st < nst; ++st) {
     const uint64_t ad = tc::smem_desc(tc::smem_u32(sF + (size_t)stage * P.f_stage_bytes), kV * 128, 1024, tc::kLayoutSW128);
     const uint64_t bd = tc::smem_desc(tc::smem_u32(sP + (size_t)stage * P.p_stage_bytes), 16, 1024, tc::kLayoutSW128);
-    if (!tc::warp_wait(&full_f[stage], phase, abort) || !tc::warp_wait(&full_p[stage], phase, abort)) return false;
+    if (!tc::mbar_wait(&full_f[stage], phase, abort) || !tc::mbar_wait(&full_p[stage], phase, abort)) return false;
     tc::tc_fence_after();
 #pragma unroll
     for (int kk = 0; kk < kV / 16; ++kk) {
@@ -74,13 +75,11 @@ __device__ __forceinline__ bool issue(const TcProjParams& P, const TcItem& item,
         if (m >= fg) break;
         const uint64_t a = ad + ((m * 2 * kV * 128 + kk * 2048) >> 4), b = bd + ((kk * 32) >> 4);
         const uint32_t d = tmem_base + (uint32_t)m * cols;
-        if (lead) {
-          tc::mma_bf16(d, a, b, idesc, (st | kk) != 0 ? 1u : 0u);
-          if (!kMerged) tc::mma_bf16(d, a, b + lo, idesc, 1u);
-        }
+        tc::mma_bf16(d, a, b, idesc, (st | kk) != 0 ? 1u : 0u);
+        if (!kMerged) tc::mma_bf16(d, a, b + lo, idesc, 1u);
       }
     }
-    if (lead) tc::mma_commit(&empty[stage]);
+    tc::mma_commit(&empty[stage]);
     if (++stage == (uint32_t)P.stages) { stage = 0; phase ^= 1; }
   }
   return true;
@@ -172,35 +171,37 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    uint32_t stage = 0, phase = 0, acc_phase = 0;
-    for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
-      const TcItem item = P.items[it];
-      if (!tc::warp_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
-      tc::tc_fence_after();
-      const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
-      bool ok;
-      if constexpr (kStageV == 32) {
-        ok = item.fg == 2 ? issue<32, 2, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
-                          : issue<32, 0, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
-      } else if (tc_merged(item.fg, item.npad)) {
-        ok = item.fg == 1   ? issue<64, 1, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
-             : item.fg == 2 ? issue<64, 2, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
-                            : issue<64, 0, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
-      } else {
-        ok = issue<64, 0, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
+    if (lane == 0) {
+      uint32_t stage = 0, phase = 0, acc_phase = 0;
+      for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
+        const TcItem item = P.items[it];
+        if (!tc::mbar_wait(acc_empty, acc_phase ^ 1, abort_flag)) break;
+        tc::tc_fence_after();
+        const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
+        bool ok;
+        if constexpr (kStageV == 32) {
+          ok = item.fg == 2 ? issue_by_one_thread<32, 2, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
+                            : issue_by_one_thread<32, 0, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
+        } else if (tc_merged(item.fg, item.npad)) {
+          ok = item.fg == 1   ? issue_by_one_thread<64, 1, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
+               : item.fg == 2 ? issue_by_one_thread<64, 2, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag)
+                              : issue_by_one_thread<64, 0, true>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
+        } else {
+          ok = issue_by_one_thread<64, 0, false>(P, item, nst, tmem_base, sF, sP, full_f, full_p, empty, stage, phase, abort_flag);
+        }
+        if (!ok) break;
+        tc::mma_commit(acc_full);
+        acc_phase ^= 1;
       }
-      if (!ok) break;
-      if (lane == 0) tc::mma_commit(acc_full);
-      acc_phase ^= 1;
     }
   } else {
     // ------------------------------------------------------------ converters + epilogue
     const int cw = warp - 2;
     const int qs = lane & 7, csub = lane >> 3;
     uint32_t stage = 0, phase = 0, acc_phase = 0;
-    // no wait of this warp has given up. The converters meet in a barrier per stage, so a warp whose wait
-    // gave up goes through the remaining stages and their barriers without working (every other wait
-    // then ends at once) instead of leaving the others there
+    // No wait of this thread has given up. The converters meet in a barrier per stage and load TMEM
+    // together, so a thread whose wait gave up does not leave: it goes through what remains without
+    // waiting (the segment's values are void then, and reported so).
     bool ok = true;
     for (int it = P.cta_first[blockIdx.x]; it < P.cta_first[blockIdx.x + 1]; ++it) {
       const TcItem item = P.items[it];
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
       const int nst = (int)((item.v1 - item.v0 + kStageV - 1) / kStageV);
       const int kb = (item.npad + 31) / 32;
       for (int st = 0; st < nst; ++st) {
-        ok = ok && tc::warp_wait(&full_f[stage], phase, abort_flag);
+        if (ok) ok = tc::mbar_wait(&full_f[stage], phase, abort_flag);
         uint8_t* tile = sP + (size_t)stage * P.p_stage_bytes;
         const float* mst = sM + (size_t)stage * kStageV;
         const int64_t vbase = item.v0 + (int64_t)st * kStageV;
@@ -268,9 +269,10 @@ __global__ void __launch_bounds__(kThreads, 1) project_tc_kernel(TcProjParams P)
         if (++stage == (uint32_t)S) { stage = 0; phase ^= 1; }
       }
       // epilogue: accumulators -> this item's partial A (k x stride, row-major)
-      ok = ok && tc::warp_wait(acc_full, acc_phase, abort_flag);
+      if (ok) ok = tc::mbar_wait(acc_full, acc_phase, abort_flag);
+      __syncwarp();
       tc::tc_fence_after();
-      if (ok) {
+      {
         const int quarter = warp & 3, half = cw >> 2;
         const int stride = item.fg * 128;
         float* part = P.ws + item.part_off;

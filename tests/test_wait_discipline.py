@@ -1,7 +1,7 @@
 """Bounded waits of the kernels whose warps have roles, read from their sources: a wait that gives up
 must not split a warp in front of a warp-collective instruction (TMEM access, barrier) or leave other
 warps in a barrier that no longer fills. So a wait by a whole warp goes through warp_wait, a plain
-mbar_wait stands in a branch of one thread, and warps that meet in a barrier of their role do not leave
+mbar_wait stands in a branch of one thread or only sets a flag of its thread, and warps that meet in a barrier of their role do not leave
 their loop in between: either the barrier carries the outcome of their waits, or no wait jumps out."""
 import os
 import re
@@ -11,12 +11,13 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2604_10377_gb300", "csrc")
 ROLES = ["k_project_tc.cu", "k_project_tc32.cu", "k_project_bwd_tc.cu", "k_project_bwd_tc32.cu", "k_gradfeat.cu"]
-ONE_THREAD = re.compile(r"\b(lane|tid|threadIdx\.x) == 0\b")
+ONE_THREAD = re.compile(r"\b(lane|tid|threadIdx\.x) == 0\b|\bissue_by_one_thread\(")
 
 
 def _enclosing_blocks(src):
     """For every plain wait: its line number and the headers of the braces around it."""
     src = re.sub(r"//[^\n]*", "", src)
+    src = re.sub(r"\bif \(ok\) ok = tc::mbar_wait", "keep_going", src)     # no branch depends on the outcome
     stack, start, found = [], 0, []
     for m in re.finditer(r"[{};]|\bmbar_wait(_cluster)?\(", src):
         t = m.group()
