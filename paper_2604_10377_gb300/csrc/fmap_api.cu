@@ -103,6 +103,7 @@ struct Plan {
   AdjTcPlan adj;
   AdjTcPlan loss_tc;        // the training loss's GEMMs on the same kernel (E, then dL/dC)
   int adj_tile = 32, loss_tile = 32;   // and the tiles of both on the CUDA cores
+  bool hi_gram = false;     // some pair's G takes the double-float sums
   bool row_grads = false;   // some pair has per-row lambda gradients to write
   fmap_sizes sizes{};
 };
@@ -191,6 +192,7 @@ int32_t make_plan(const fmap_options& opt, const fmap_shape_desc* shapes, int32_
     pd.dlam_rows = q.lambda_rows ? q.d_lambda_rows : nullptr;
     if (pd.dlam_rows) P.row_grads = true;
     pd.hi_gram = sx.k >= opt.hi_gram_min_k ? 1 : 0;
+    if (pd.hi_gram) P.hi_gram = true;
     pd.c_off = P.c_off[p];
     P.c_off[p + 1] = P.c_off[p] + (int64_t)sy.k * sx.k;
   }
@@ -1004,7 +1006,7 @@ int32_t fmap_solve(fmap_batch* b, const float* a, float* c_out, void* saved, int
   if (e != cudaSuccess) return cuda_fail(e, "status_clear");
   {
     TimedScope ts(b, FMAP_KIND_GRAM, st);
-    e = launch_gram(b->dev, b->plan.max_k, a, w, st);
+    e = launch_gram(b->dev, b->plan.max_k, b->plan.max_d, b->plan.hi_gram, a, w, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "gram");
   for (const auto& g : b->plan.groups) {
@@ -1051,7 +1053,7 @@ int32_t adjoint_impl(fmap_batch* b, const float* d_c, const float* a, const floa
   for (const PairDev& pd : b->plan.pairs) need_g = need_g || pd.fac_off < 0;
   if (need_g) {
     TimedScope ts(b, FMAP_KIND_GRAM, st);
-    e = launch_gram(b->dev, b->plan.max_k, a, w, st, /*with_r=*/false);
+    e = launch_gram(b->dev, b->plan.max_k, b->plan.max_d, b->plan.hi_gram, a, w, st, /*with_r=*/false);
   }
   if (e != cudaSuccess) return cuda_fail(e, "gram");
   for (const auto& g : b->plan.groups) {

@@ -197,7 +197,8 @@ __host__ __device__ constexpr int tc_red_subs(int parts) { return parts < 16 ? 1
 // ---- launchers (each enqueues on `st`; return cudaError_t of the launch) ----
 // with_r = false computes G only (the adjoint solves never read R)
 cudaError_t gram_set_smem();
-cudaError_t launch_gram(const BatchDev& b, int max_k, const float* a, float* ws, cudaStream_t st,
+// (hi_gram: some pair takes the double-float sums)
+cudaError_t launch_gram(const BatchDev& b, int max_k, int max_d, bool hi_gram, const float* a, float* ws, cudaStream_t st,
                         bool with_r = true);
 
 struct SolveGroup {

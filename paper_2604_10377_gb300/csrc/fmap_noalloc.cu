@@ -160,7 +160,7 @@ extern "C" FMAP_API int32_t fmap_solve_pair_noalloc(const float* a_x, const floa
   b.feat_bf16 = 0;
   b.ir_steps = ir_steps;
   if (launch_status_clear(status, 1, st) != cudaSuccess) return FMAP_ERR_CUDA;
-  if (launch_gram(b, k, a_x, scratch, st) != cudaSuccess) return FMAP_ERR_CUDA;
+  if (launch_gram(b, k, d, hi, a_x, scratch, st) != cudaSuccess) return FMAP_ERR_CUDA;
   SolveGroup g{};
   g.first = 0;
   g.count = k;

@@ -221,15 +221,20 @@ cudaError_t gram_set_smem() {
   return cudaFuncSetAttribute(gram_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GramSmem<8>));
 }
 
-cudaError_t launch_gram(const BatchDev& b, int max_k, const float* a, float* ws, cudaStream_t st, bool with_r) {
+cudaError_t launch_gram(const BatchDev& b, int max_k, int max_d, bool hi_gram, const float* a, float* ws,
+                        cudaStream_t st, bool with_r) {
   if (b.n_pairs <= 0) return cudaSuccess;
-  // 4 groups, or 8 where the batch has not two tiles of G per SM and its k can reach the
-  // double-float sums (the chain of a tile then bounds the launch: 4 pairs of k = 200, d = 512
-  // 0.037 ms against 0.060; 8 pairs of k = 100, d = 384, FP32 sums, 0.0185 against 0.0164)
-  // G first: its double-float tiles (k >= hi_gram_min_k) are the longest
+  // Four groups, or eight where a tile's chain bounds the launch: double-float sums while G has at most a
+  // tile per SM, FP32 sums of 256 features or more while all tiles together leave a third of the SMs
+  // idle. us, four / eight: one, 4, 8 pairs of k = 200, d = 512 37 / 33, 60 / 40, 64 / 68, one, 2, 4 of k = 300
+  // 41 / 33, 60 / 41, 64 / 68, 4 of k = 64, d = 384 with double-float sums 30 / 27, 16 of k = 100 47 / 47; FP32
+  // sums, d = 512, one, 2, 4 of k = 199 14.2 / 13.4, 18.4 / 18.6, 24 / 27, one and 8 of k = 100 14.1 / 13.1,
+  // 18.5 / 20.3, one of k = 100, d = 128 8.2 / 8.6.
+  // G first: its double-float tiles are the longest
   const int nt = (max_k + kT - 1) / kT;
   dim3 grid(nt * nt, b.n_pairs, with_r ? 2 : 1);
-  if (max_k > 128 && (int64_t)nt * (nt + 1) / 2 * b.n_pairs < 2 * 152)
+  const int64_t g_tiles = (int64_t)nt * (nt + 1) / 2 * b.n_pairs, tiles = g_tiles + (with_r ? (int64_t)nt * nt * b.n_pairs : 0);
+  if (hi_gram ? g_tiles <= 152 : (tiles <= 100 && max_d >= 256))
     gram_kernel<8><<<grid, 512, sizeof(GramSmem<8>), st>>>(b, a, ws);
   else
     gram_kernel<4><<<grid, 256, sizeof(GramSmem<4>), st>>>(b, a, ws);
