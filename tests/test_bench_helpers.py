@@ -2,6 +2,7 @@
 for the kernel sources it was captured on, and the algorithmic work per step follows the
 sizes of the batch."""
 import hashlib
+import json
 import os
 import sys
 import types
@@ -93,3 +94,28 @@ def test_config_sizes_match_the_drawn_shapes():
     wl = synth.make_config(1, pairs=[0, 5, 31], n_scale=1.0)
     for j, p in enumerate([0, 5, 31]):
         assert sizes[p] == (wl.shapes[2 * j].n, wl.shapes[2 * j + 1].n, wl.shapes[2 * j].k)
+
+
+def test_result_line_is_short_and_details_keep_the_rest():
+    """The line that carries the headline stays well inside the end of the output that a reader keeps."""
+    roof = {"kernel": "solve", "bound": "alu", "achieved": 1.2345678901234567, "peak": 77.12345678901234, "unit": "TFLOP/s",
+            "frac": 0.123456789012345, "traffic": 1234567890123, "algorithmic_bytes": 1234567890,
+            "peak_source": "measured FP32 FMA loop on this GPU (fmap_peak_loop)"}
+    kernels = {f"kind_{i}": {"ms_per_step": 1.2345678901234567, "launches_per_step": 6.0} for i in range(10)}
+    acc = {"pairs": 8, "pairs_sampled": list(range(248, 256)), "C_rel_fro_max": 1.68e-05, "reference": "FP64 oracle on the same inputs"}
+    sub = {"value": 1.0, "roofline": roof, "roofline_other": {f"k{i}": roof for i in range(4)}, "kernels": kernels, "accuracy": acc}
+    line = {"metric": bench.METRIC, "value": 31880.0, "unit": "pairs/s", "n_gpus": 1, "steps": 20, "warmup": 5,
+            "ms_per_step": 8.03, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16/f32",
+            "data": "synthetic", "config": {"workload": bench.WORKLOADS[4]}, "roofline": roof, "kernels": kernels,
+            "roofline_other": sub["roofline_other"], "gpu_launches": 400, "accuracy": acc, "clocks": {"sm_mhz": 2070},
+            "e2e": {"value": 5010.0}, "cpu_baseline": {"sample": "k=" + str([200] * 32)}, "torch_restatement": {"value": 1905.0},
+            "autotune": {"trials": [{"tuning": {"proj_max_stages": 4}, "ms": 8.123456789}] * 19}, "peaks_measured": {"fp32_fma": 77.4},
+            "workloads": {str(i): sub for i in range(4)}, "gradient_features": {"variants": {"A": roof, "B": roof}}}
+    short, details = bench.split_line(dict(line))
+    assert len(json.dumps(short)) < 6000
+    assert {"metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+            "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline"} <= set(short)
+    merged = dict(short)
+    for d in details:
+        merged.update({k: v for k, v in d.items() if k != "detail"})
+    assert merged == line
