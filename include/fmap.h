@@ -76,9 +76,9 @@ typedef struct fmap_options {
     int32_t proj_seg_max_v;     /* tensor-core projection of BF16 features: longest vertex segment
                                    accumulated in TMEM before a partial is written, multiple of
                                    64 in 2048..16384 (default 8192); FP32 features always use
-                                   512 (accuracy of the three TF32 passes) */
-    int32_t bwd_group_features; /* tensor-core backward projection: features per CTA group,
-                                   64 or 128 (default 128) */
+                                   2048, or 512 where one accumulator takes all products */
+    int32_t bwd_group_features; /* tensor-core backward projection of BF16 features: features per
+                                   CTA, 64 or 128 (default 128); FP32 features always take 64 */
     int32_t bwd_chunk_v;        /* tensor-core backward projection: largest vertex chunk of a work
                                    item, multiple of 128 in 1024..65536 (default 8192; BF16
                                    features round it up to 256) */
@@ -95,8 +95,7 @@ typedef struct fmap_options {
     int32_t adjoint_kernel;     /* W = Gamma^T C + C^T Gamma, dA_x = Gamma^T A_y - W A_x, dA_y = Gamma A_x,
                                    and the training loss's E = C C^T - I, dL/dC = 4 E C + 2 (C - C_gt):
                                    1 tensor cores (three TF32 passes), 2 CUDA cores (FP32 FMA tiles);
-                                   0 the built-in choice, by the arithmetic of the batch against its
-                                   longest reduction */
+                                   0 the built-in choice, by the time either would take */
     int32_t adjoint_features;   /* tensor-core adjoint GEMMs: output columns per CTA, 64, 128 or 256
                                    (default 128, or 64 below two dA_x tiles per SM) */
     int32_t adjoint_stages;     /* tensor-core adjoint GEMMs: shared-memory stages per CTA, 1 or 2

@@ -82,9 +82,9 @@ struct Plan {
   int64_t da_int_off = 0;
   int64_t loss_part_off = 0;
   // tensor-core projection
-  bool tc32 = false;      // FP32 features: three-pass TF32 kernel
+  bool tc32 = false;      // FP32 features: three BF16 parts of each operand
   bool tc_bwd = false;    // backward projection on the tensor cores (BF16 features: CTA pairs)
-  bool tc_bwd32 = false;  // backward projection on the tensor cores (FP32 features: three TF32 passes)
+  bool tc_bwd32 = false;  // backward projection on the tensor cores (FP32 features: three BF16 parts)
   std::vector<TcItem> tc_items;
   int proj_ctas = kTcCtas;             // persistent CTAs of the forward projection
   int bwd_ctas = kTcCtas;              // and of the backward projection

@@ -207,7 +207,7 @@ struct SolveGroup {
   int32_t kmax;      // largest k in the group
   int32_t threads;
   int32_t no_g_copy; // 1: no shared-memory copy of G for the refinement residual (the residual
-                     // then reads G from L2); 0: the built-in rule, a copy for k <= 128
+                     // then reads G from L2); 0: the built-in rule, a copy for k <= 100
 };
 
 enum SolveMode { kSolveForward = 0, kSolveAdjoint = 1 };

@@ -31,8 +31,8 @@
 namespace fmap {
 namespace {
 
-// Rounds of 128 columns that cover a row of G in the refinement residual.
-constexpr int kResRounds = (kMaxK + 127) / 128;
+// Rounds of 128 columns that cover a row of G in the refinement residual of chol_solve_kernel.
+constexpr int kResRounds = (kSolveBounds[4] + 127) / 128;
 
 // Floats of one factor: the packed rows plus the Q inverse diagonal blocks.
 __host__ __device__ __forceinline__ int factor_floats(int Q) { return 32 * Q * (Q + 2) + 64 * Q; }
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(NT, (NT >= 256 ? 2 : (NT >= 128 ? 4 : 8)))
   if (tid == 0) tc::bulk_wait_group_read0();   // the factor has left shared memory
 }
 
-// ---- k > 128: the trailing matrix in registers -------------------------------------
+// ---- above k = 100 (but 201 .. 208): the trailing matrix in registers ----------------
 // Pairs of column halves of a panel in shared memory: entry (row a, column c) of the
 // current panel is at c * 2 * half + ((a >> 2) & 1) * half + 4 * (a >> 3) + (a & 3), so
 // that consecutive 8-row blocks read consecutive float4 and, with half = 16 mod 32, the
@@ -1064,7 +1064,7 @@ __device__ __forceinline__ float residual_piece(const Load& entry, const float* 
   return p[0] + __shfl_xor_sync(0xffffffffu, p[0], 16);
 }
 
-// Row systems with k > 128: the factorisation above, then the solves of chol_solve_kernel.
+// Row systems of those sizes: the factorisation above, then the solves of chol_solve_kernel.
 template <int OW, int RW, int kSlots, int kMinBlocks>
 __global__ void __launch_bounds__(32 * (1 + OW + RW), kMinBlocks)
     chol_reg_kernel(BatchDev b, const int2* systems, int first, int count, int mode, const float* rhs_flat,
@@ -1232,7 +1232,7 @@ size_t chol_reg_smem_bytes(int kmax) {
 }
 
 // Launches for k <= kGsMaxK reserve a copy of G (k x gram_ld(k) floats) after the vectors.
-constexpr int kGsMaxK = 128;
+constexpr int kGsMaxK = kSolveBounds[1];
 
 size_t chol_smem_bytes(int kmax, bool g_copy = true) {
   const int Q = (kmax + 7) / 8, kp = 8 * Q;
@@ -1269,7 +1269,8 @@ cudaError_t solve_set_smem_limits() {
 // 32 at k = 200), shared memory against registers: k = 77 37.2 / 9.9 against 48.6 / 9.2,
 // k = 100 60.0 / 14.3 against 64.9 / 11.0, k = 104 76.5 / 20.0 against 64.5 / 11.0, k = 112
 // 81.7 / 19.5 against 71.0 / 11.0, k = 128 98.0 / 20.0 against 99.4 / 11.8, k = 200 252 / 46
-// (with an inverse in every step of its solves) against 221 / 27.
+// (with an inverse in every step of its solves) against 221 / 27. The adjoint alone would change at
+// k = 77; it takes the forward solve's kernel up to 100, a quarter of whose time it is.
 cudaError_t launch_solve(const BatchDev& b, const SolveGroup& g, const int2* systems, int mode, const float* rhs_flat,
                          float* out_flat, float* saved, int32_t* status, float* ws, cudaStream_t st) {
   if (g.count <= 0) return cudaSuccess;

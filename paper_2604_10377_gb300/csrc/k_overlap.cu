@@ -12,10 +12,10 @@
 // by HBM bandwidth. The segments are contiguous, so the flat vertex range is cut into equal
 // spans, one per warp, whatever the segment lengths (a (chunk, segment) grid leaves most of
 // its blocks without work on short segments). 4096 segments, 87 M vertices: 0.088 ms on the
-// device = 5.0 TB/s; a call with its upload of the offsets 0.117 ms, 0.181 ms with the grid. A warp finds its first segment with a 32-way search over the
-// offsets, reads four scores and four labels per lane and load (four such loads in flight),
-// and adds the counts of each segment it meets with one integer atomic per count (integer
-// sums: exact and order-independent).
+// device = 5.0 TB/s; a call with its upload of the offsets 0.117 ms, 0.181 ms with the grid. A
+// warp finds its first segment with a 32-way search over the offsets, reads four scores and four
+// labels per lane and load (four such loads in flight), and adds the counts of each segment it
+// meets with one integer atomic per count (integer sums: exact and order-independent).
 #include <stdint.h>
 
 #include "fmap_internal.cuh"

@@ -4,7 +4,7 @@
 //   dF_s (n x d, FP32) = diag(M_s) Phi_s (n x k) . dA_s (k x d)
 //
 // Same split as the FP32 forward projection: Phi and dA are exact sums of three BF16 numbers
-// each, and six of the nine products are accumulated in FP32 (what is left out is below 2^-26
+// each, and six of the nine products are accumulated in FP32 (what is left out is at most 2^-24
 // of a product).
 //
 // kind::f16 MMA, M = 128 vertices, N = up to three thirds of one group of <= 64 features, K =
@@ -23,7 +23,7 @@
 // and the hand-over of the slots. 32 shapes of n = 50000, d = 256, against Phi and its remainder in
 // shared memory, three TF32 MMAs on 64 features at a time and two images of dA^T, for which groups
 // shrank to 32 features above k = 192: k = 30 425 -> 441 us, k = 50 567 -> 508, k = 100 1022 -> 869,
-// k = 200 3132 -> 1371. One accumulator and six slots: 5 to 14% slower; the groups' items one after
+// k = 200 3132 -> 1371 (k = 30 with store boxes of 16 features: 515). One accumulator and six slots: 5 to 14% slower; the groups' items one after
 // the other instead of chunk by chunk: up to 3% slower at k <= 64, the same above.
 // Waits are bounded like the other tensor-core kernels'.
 #include "fmap_internal.cuh"
