@@ -19,8 +19,8 @@
 // A vertex's row of X is read about seven times among its neighbours: 128 vertices times 64 bytes
 // keep the rows in hand inside L1, where gathering whole 512-byte rows read every one of them
 // from L2 before a tile's products could start (64 shapes, 1.06 M vertices, D = 128: 1.215 ms a
-// call, 0.607 this way). What bounds it now is the load pipe of L1 (about 14k wavefronts of 23k
-// cycles per tile: eight rows of X to a load instruction, 32 output rows to a store).
+// call, 0.600 this way). What bounds it now is the data pipe of L1 (14.8k wavefronts in the 21.0k
+// cycles of a tile: eight rows of X to a load instruction, 32 output rows to a store).
 // The x, y tile is the MMA operand and the epilogue's input, so a tile's gather starts
 // after the previous tile's epilogue. Waits are bounded; a wait that gives up, or a CSR
 // index out of range, sets the caller's status word.

@@ -378,11 +378,6 @@ __device__ __forceinline__ bool named_barrier_or(int id, int nthreads, bool x) {
   return r != 0;
 }
 
-// Counts the calling warp in without waiting.
-__device__ __forceinline__ void named_barrier_arrive(int id, int nthreads) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
 // Arrive on `bar` once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
